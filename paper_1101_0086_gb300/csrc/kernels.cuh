@@ -914,13 +914,35 @@ template <typename T> struct ScanParams {
     DbgRange dbg;  // checked range of the debug build
 };
 
-// Adds this block's sums to link l's accumulators; the last block of the
-// level closes the level (comparison with the previous one, reset).
+// One thread adds a block's sums to a link's accumulators; the last of the
+// level's nblk blocks closes the level (comparison with the previous one, reset).
+__device__ __forceinline__ void conv_level(ConvState* cs, unsigned int* err, double sd, double sp, int level,
+                                           int last_level, double floor_rel, unsigned nblk) {
+    atomicAdd(&cs->acc_d, sd);
+    atomicAdd(&cs->acc_p, sp);
+    __threadfence();
+    if (atomicAdd(&cs->count, 1u) != nblk - 1) return;
+    __threadfence();
+    volatile ConvState* v = cs;
+    const double ad = v->acc_d, ap = v->acc_p;
+    const double rel = ap > 0.0 ? sqrt(ad / ap) : 0.0;
+    if (level > 0) {
+        const double q = v->prev_rel > 0.0 ? rel / v->prev_rel : (rel > 0.0 ? 1e300 : 0.0);
+        if (q > v->worst) v->worst = q;
+        if (!(rel < v->prev_rel) && rel > floor_rel) atomicOr(err, ERR_DIVERGED);
+    }
+    v->prev_rel = level == last_level ? 0.0 : rel;
+    v->acc_d = 0.0;
+    v->acc_p = 0.0;
+    v->count = 0u;
+}
+
+// The block's sums of d2 and p2 (every thread of the block calls) into link
+// l's accumulators.
 __device__ __forceinline__ void conv_close(ConvState* cs, unsigned int* err, double d2, double p2, int level,
                                            int last_level, double floor_rel, unsigned nblk) {
     __shared__ double red[2][32];  // one entry per warp (up to 1024 threads)
-    __shared__ bool last_block;
-    // warp sums, then the block's 8 warp sums by thread 0
+    // warp sums, then the block's warp sums by thread 0
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         d2 += __shfl_xor_sync(0xffffffffu, d2, o);
@@ -938,33 +960,10 @@ __device__ __forceinline__ void conv_close(ConvState* cs, unsigned int* err, dou
             sd += red[0][i];
             sp += red[1][i];
         }
-        atomicAdd(&cs->acc_d, sd);
-        atomicAdd(&cs->acc_p, sp);
-        __threadfence();
-        last_block = atomicAdd(&cs->count, 1u) == nblk - 1;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && last_block) {
-        __threadfence();
-        volatile ConvState* v = cs;
-        const double sd = v->acc_d, sp = v->acc_p;
-        const double rel = sp > 0.0 ? sqrt(sd / sp) : 0.0;
-        if (level > 0) {
-            const double q = v->prev_rel > 0.0 ? rel / v->prev_rel : (rel > 0.0 ? 1e300 : 0.0);
-            if (q > v->worst) v->worst = q;
-            if (!(rel < v->prev_rel) && rel > floor_rel) atomicOr(err, ERR_DIVERGED);
-        }
-        v->prev_rel = level == last_level ? 0.0 : rel;
-        v->acc_d = 0.0;
-        v->acc_p = 0.0;
-        v->count = 0u;
+        conv_level(cs, err, sd, sp, level, last_level, floor_rel, nblk);
     }
 }
 
-// Frequency k of link l (one thread each; a block of consecutive
-// frequencies, nblk blocks per link).  N is a multiple of the block size (a
-// power of two >= 256), so every thread has a frequency and takes part in
-// the block reduction of the increment check.
 // 8-byte global -> shared copy (cp.async.ca) and its commit / wait groups
 __device__ __forceinline__ void cp_async8(void* dst, const void* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
@@ -975,6 +974,66 @@ template <int N> __device__ __forceinline__ void cp_async_wait_group() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
+// What follows the sums at one frequency (position i, natural index k) of
+// link l, D = (sx, sy) being the trapezoid sum of Eq. (6) at node M: the
+// Picard increment check, and at the last level step 7 (mode 1) or psi_M
+// (mode 2).  BLOCK: every thread of the block calls, and the check's sums go
+// through a block reduction; else one whole warp of the block calls, and its
+// sums are the block's.
+template <typename T, bool CG, bool BLOCK>
+__device__ __forceinline__ void scan_node_m(const ScanParams<T>& p, int l, long long i, long long k, cx<T> p0, double sx,
+                                            double sy, unsigned nblk) {
+    typedef cx<T> C;
+    const long long lo = (long long)l * p.N;
+    if (p.conv) {
+        // Picard increment at node M against the previous level's D
+        double dx = sx, dy = sy;
+        if (p.level > 0) {
+            const float2 d0 = MPA_DBG_OK(p.dbg, p.dprev + lo + i, sizeof(float2)) ? ldx<CG>(p.dprev + lo + i)
+                                                                                 : make_float2(0.f, 0.f);
+            dx -= (double)d0.x;
+            dy -= (double)d0.y;
+        }
+        if (p.level < p.n_iter - 1 && MPA_DBG_OK(p.dbg, p.dprev + lo + i, sizeof(float2)))
+            p.dprev[lo + i] = make_float2((float)sx, (float)sy);
+        const double px = (double)p0.x - sy, py = (double)p0.y + sx;
+        double d2 = dx * dx + dy * dy, p2 = px * px + py * py;
+        if constexpr (BLOCK) {
+            conv_close(p.conv + l, p.err, d2, p2, p.level, p.n_iter - 1, p.floor_rel, nblk);
+        } else {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                d2 += __shfl_xor_sync(0xffffffffu, d2, o);
+                p2 += __shfl_xor_sync(0xffffffffu, p2, o);
+            }
+            if ((threadIdx.x & 31) == 0)
+                conv_level(p.conv + l, p.err, d2, p2, p.level, p.n_iter - 1, p.floor_rel, nblk);
+        }
+    }
+    if (p.mode == 0) return;
+    const double2 s0 = MPA_DBG_OK(p.dbg, p.state + lo + k, sizeof(double2)) ? ldx<CG>(p.state + lo + k)
+                                                                          : make_double2(0.0, 0.0);
+    const double2 psiM = make_double2(s0.x - sy, s0.y + sx);
+    if (p.mode == 2) {
+        p.out[lo + k] = psiM;  // the caller's buffer (mpa_interval), outside the workspace
+        return;
+    }
+    // step 7 and the lumped gain
+    NodeC nodeM{};
+    if (MPA_DBG_OK(p.dbg, p.loff + l, sizeof(int)) && MPA_DBG_OK(p.dbg, p.nodes + p.loff[l] + p.M, sizeof(NodeC)))
+        nodeM = p.nodes[p.loff[l] + p.M];
+    const double2 ph = expi_turns<double>(phase_q64(signed_k(k, p.N), nodeM));
+    const double g = nodeM.pre * (MPA_DBG_OK(p.dbg, p.gain + l, sizeof(double)) ? p.gain[l] : 0.0);
+    const double2 a = make_double2(g * (psiM.x * ph.x - psiM.y * ph.y), g * (psiM.x * ph.y + psiM.y * ph.x));
+    if (MPA_DBG_OK(p.dbg, p.state + lo + k, sizeof(double2))) p.state[lo + k] = a;
+    if (MPA_DBG_OK(p.dbg, p.psi0c_out + lo + k, sizeof(C))) p.psi0c_out[lo + k] = mkc((T)a.x, (T)a.y);
+    if (!(isfinite(a.x) && isfinite(a.y))) atomicOr(p.err, ERR_NONFINITE);
+}
+
+// Frequency k of link l (one thread each; a block of consecutive
+// frequencies, nblk blocks per link).  N is a multiple of the block size (a
+// power of two >= 256), so every thread has a frequency and takes part in
+// the block reduction of the increment check.
 // S > 0 (FP32 only): the thread's V_j travel S nodes ahead through its own S
 // shared-memory slots (ring[slot * blockDim.x + threadIdx.x]) by 8-byte
 // cp.async, one commit group per node, so the bytes in flight do not cost
@@ -1059,38 +1118,7 @@ __device__ __forceinline__ void scan_freq(const ScanParams<T>& p, int l, long lo
     // D = R_M - V_M/2 at node M in FP64 (psi_M = psi_0 + i D)
     const double sx = ((double)rx - (double)cxx) - 0.5 * (double)vl.x;
     const double sy = ((double)ry - (double)cyy) - 0.5 * (double)vl.y;
-    if (p.conv) {
-        // Picard increment at node M against the previous level's D
-        double dx = sx, dy = sy;
-        if (p.level > 0) {
-            const float2 d0 = MPA_DBG_OK(p.dbg, p.dprev + lo + i, sizeof(float2)) ? ldx<CG>(p.dprev + lo + i)
-                                                                                 : make_float2(0.f, 0.f);
-            dx -= (double)d0.x;
-            dy -= (double)d0.y;
-        }
-        if (p.level < p.n_iter - 1 && MPA_DBG_OK(p.dbg, p.dprev + lo + i, sizeof(float2)))
-            p.dprev[lo + i] = make_float2((float)sx, (float)sy);
-        const double px = (double)p0.x - sy, py = (double)p0.y + sx;
-        conv_close(p.conv + l, p.err, dx * dx + dy * dy, px * px + py * py, p.level, p.n_iter - 1, p.floor_rel, nblk);
-    }
-    if (p.mode == 0) return;
-    const double2 s0 = MPA_DBG_OK(p.dbg, p.state + lo + k, sizeof(double2)) ? ldx<CG>(p.state + lo + k)
-                                                                          : make_double2(0.0, 0.0);
-    const double2 psiM = make_double2(s0.x - sy, s0.y + sx);
-    if (p.mode == 2) {
-        p.out[lo + k] = psiM;  // the caller's buffer (mpa_interval), outside the workspace
-        return;
-    }
-    // step 7 and the lumped gain
-    NodeC nodeM{};
-    if (MPA_DBG_OK(p.dbg, p.loff + l, sizeof(int)) && MPA_DBG_OK(p.dbg, p.nodes + p.loff[l] + p.M, sizeof(NodeC)))
-        nodeM = p.nodes[p.loff[l] + p.M];
-    const double2 ph = expi_turns<double>(phase_q64(signed_k(k, p.N), nodeM));
-    const double g = nodeM.pre * (MPA_DBG_OK(p.dbg, p.gain + l, sizeof(double)) ? p.gain[l] : 0.0);
-    const double2 a = make_double2(g * (psiM.x * ph.x - psiM.y * ph.y), g * (psiM.x * ph.y + psiM.y * ph.x));
-    if (MPA_DBG_OK(p.dbg, p.state + lo + k, sizeof(double2))) p.state[lo + k] = a;
-    if (MPA_DBG_OK(p.dbg, p.psi0c_out + lo + k, sizeof(C))) p.psi0c_out[lo + k] = mkc((T)a.x, (T)a.y);
-    if (!(isfinite(a.x) && isfinite(a.y))) atomicOr(p.err, ERR_NONFINITE);
+    scan_node_m<T, CG, true>(p, l, i, k, p0, sx, sy, nblk);
 }
 
 // Nodes in flight per thread of the FP32 scan (shared-memory slots; 0: the
@@ -1108,6 +1136,101 @@ __global__ void __launch_bounds__(256) scan_kernel(const ScanParams<T> p) {
                                              ring);
     } else {
         scan_freq<T, false>(p, blockIdx.y, (long long)blockIdx.x * blockDim.x + threadIdx.x, gridDim.x);
+    }
+}
+
+// The scan with the nodes of a frequency split over the block: 32 frequencies
+// (lanes) x SCS_W warps, warp w taking a run of up to SCS_C consecutive nodes
+// of each panel of nodes.  A thread loads its run into registers at once and
+// sums it; the runs' sums are combined through shared memory (compensated in
+// FP32 like the sums themselves), and the thread adds its exclusive prefix to
+// the run's partial sums.  A short link leaves scan_kernel with few warps
+// that each walk all M nodes one after another (N = 2^12: 16 blocks on 152
+// SMs, bound by L2 latency); here every node of a panel is in flight at once.
+// Eight warps at 64 registers: four blocks an SM, whose load, sum and store
+// phases overlap (16 warps at 64 registers 52 us, 101 registers 66 us, these
+// 43 us on a level of 2^14 x 801 nodes; scan_kernel 80 us).
+constexpr int SCS_W = 8;
+template <typename T>
+__global__ void __launch_bounds__(32 * SCS_W, sizeof(T) == 4 ? 4 : 2) scan_split_kernel(const ScanParams<T> p) {
+    typedef cx<T> C;
+    constexpr bool F32 = sizeof(T) == 4;
+    constexpr int SCS_C = F32 ? 16 : 8;         // nodes a thread holds
+    __shared__ C ps[SCS_W][32], pc[SCS_W][32];  // the runs' sums and compensations
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, l = blockIdx.y;
+    const long long i = (long long)blockIdx.x * 32 + lane;
+    const long long lo = (long long)l * p.N;
+    C* psi = p.psi + lo * (p.M + 1) + i;
+    const long long k = p.tile_logG > 0 ? tile_to_natural(i, p.tile_logG, p.tile_logL, p.N) : i;
+    const C zero = mkc(T(0), T(0));
+    const C v0 = MPA_DBG_OK(p.dbg, psi, sizeof(C)) ? *psi : zero;
+    const C p0 = MPA_DBG_OK(p.dbg, p.psi0c + lo + k, sizeof(C)) ? p.psi0c[lo + k] : zero;
+    // equal runs: as few panels as the registers allow, nodes spread evenly over them
+    const int panels = (p.M + SCS_W * SCS_C - 1) / (SCS_W * SCS_C);
+    const int run = (p.M + SCS_W * panels - 1) / (SCS_W * panels);
+    C r = mkc(T(0.5) * v0.x, T(0.5) * v0.y), c = zero;  // sum before the panel and its compensation
+    for (int jb = 1; jb <= p.M; jb += SCS_W * run) {
+        const int j0 = jb + w * run;
+        const int n = p.M + 1 - j0 < run ? p.M + 1 - j0 : run;  // nodes of this thread's run (<= 0: none)
+        C* a = psi + (long long)j0 * p.N;
+        C v[SCS_C];
+#pragma unroll
+        for (int u = 0; u < SCS_C; ++u)
+            v[u] = u < n && MPA_DBG_OK(p.dbg, a + (long long)u * p.N, sizeof(C)) ? a[(long long)u * p.N] : zero;
+        // v[u] <- (sum of the run before node u) + V_u / 2
+        C s = zero, sc = zero, vl = zero;
+#pragma unroll
+        for (int u = 0; u < SCS_C; ++u) {
+            const C x = v[u];
+            if (u < n) vl = x;
+            v[u] = mkc((F32 ? s.x - sc.x : s.x) + T(0.5) * x.x, (F32 ? s.y - sc.y : s.y) + T(0.5) * x.y);
+            if constexpr (F32) {
+                kahan_add(s.x, sc.x, x.x);
+                kahan_add(s.y, sc.y, x.y);
+            } else {
+                s.x += x.x;
+                s.y += x.y;
+            }
+        }
+        if (jb > 1) __syncthreads();  // the previous panel's sums have been read
+        ps[w][lane] = s;
+        if constexpr (F32) pc[w][lane] = sc;
+        __syncthreads();
+        C mr = r, mc = c;  // sum before this thread's run
+#pragma unroll
+        for (int q = 0; q < SCS_W; ++q) {
+            if (q == w) {
+                mr = r;
+                mc = c;
+            }
+            const C t = ps[q][lane];
+            if constexpr (F32) {
+                const C tc = pc[q][lane];
+                kahan_add(r.x, c.x, t.x);
+                kahan_add(r.y, c.y, t.y);
+                c.x += tc.x;
+                c.y += tc.y;
+            } else {
+                r.x += t.x;
+                r.y += t.y;
+            }
+        }
+        if (p.mode == 0) {
+            const C b = F32 ? mkc(mr.x - mc.x, mr.y - mc.y) : mr;
+#pragma unroll
+            for (int u = 0; u < SCS_C; ++u)
+                if (u < n && MPA_DBG_OK(p.dbg, a + (long long)u * p.N, sizeof(C)))
+                    a[(long long)u * p.N] = mkc(p0.x - (b.y + v[u].y), p0.y + (b.x + v[u].x));
+        }
+        if (n > 0 && j0 + n == p.M + 1) {  // the warp of node M
+            // D = R_M - V_M/2 at node M in FP64, R_M = the sum before the run + the run
+            double sx = (double)mr.x + (double)s.x, sy = (double)mr.y + (double)s.y;
+            if constexpr (F32) {
+                sx -= (double)mc.x + (double)sc.x;
+                sy -= (double)mc.y + (double)sc.y;
+            }
+            scan_node_m<T, false, false>(p, l, i, k, p0, sx - 0.5 * (double)vl.x, sy - 0.5 * (double)vl.y, gridDim.x);
+        }
     }
 }
 

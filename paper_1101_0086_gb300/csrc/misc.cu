@@ -181,11 +181,21 @@ void prof_reset() {
 
 static unsigned blocks_for(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
+// Frequencies (N x links) up to which a scan splits its nodes over the block
+// (scan_split_kernel).  Measured, us a launch, split / unsplit: FP32, 143
+// nodes: 2^12 13.5 / 20.9, 2^14 17.7 / 20.6, 2^15 24.5 / 21.7; 801 nodes:
+// 2^12 21 / 63, 2^14 43 / 80.  FP64 is bound by its adds, which the split
+// form doubles: 143 nodes 2^12 24 / 54, 2^13 37 / 54.
+template <typename T> constexpr long long scan_split_max() { return sizeof(T) == 4 ? 1ll << 14 : 1ll << 13; }
+
 template <typename T> cudaError_t scan_launch(const ScanParams<T>& p, int p_links, cudaStream_t st) {
     if (const cudaError_t eg = launch_gate()) return eg;
     const bool pr = g_prof_on.load(std::memory_order_relaxed);
     if (pr) prof_begin(st);
-    scan_kernel<T><<<dim3(blocks_for(p.N, 256), (unsigned)p_links), 256, 0, st>>>(p);
+    if (p.N * p_links <= scan_split_max<T>())
+        scan_split_kernel<T><<<dim3(blocks_for(p.N, 32), (unsigned)p_links), 32 * SCS_W, 0, st>>>(p);
+    else
+        scan_kernel<T><<<dim3(blocks_for(p.N, 256), (unsigned)p_links), 256, 0, st>>>(p);
     if (pr) {
         const double cs = (double)sizeof(cx<T>), n = (double)p.N;
         double b = ((p.M + 1) * n * cs + n * cs) * p_links;  // V_0..V_M and psi_0
