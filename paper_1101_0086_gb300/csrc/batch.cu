@@ -34,6 +34,8 @@ struct Group {
     Split sp;
     std::vector<int> links;        // batch link indices, longest first
     std::vector<NodeC> nodes;      // concatenated per-link tables
+    std::vector<ScanNode> scn;     // FP32: the scan's constants, indexed as nodes
+    size_t off_scn = 0;
     std::vector<int> loff;         // [q][active link]
     std::vector<double> gain;      // [q][active link]
     std::vector<int> active;       // links running at interval q
@@ -167,7 +169,7 @@ int run_group(mpa_batch* b, Group& g, cudaStream_t st) {
         for (long q = 0; q < g.n_int; ++q) {
             int rc = mpa_levels<T>(s, M, b->n_iter, g.active[(size_t)q], psi,
                                    g.has_work ? reinterpret_cast<cx<T>*>(b->ws + g.off_work) : nullptr, psi0c, state,
-                                   nodes, loff + (size_t)q * n, gain + (size_t)q * n, mon, 1, nullptr, st);
+                                   nodes, reinterpret_cast<const ScanNode*>(b->ws + g.off_scn), loff + (size_t)q * n, gain + (size_t)q * n, mon, 1, nullptr, st);
             if (rc) return rc;
         }
     }
@@ -286,6 +288,7 @@ int mpa_batch_create(const mpa_link* links, int32_t n_links, double L_km, int32_
             for (int i = 0; i < n; ++i)
                 n_nodes += (size_t)b->links[(size_t)g.links[(size_t)i]].n_types * ((size_t)M + 1);
             g.nodes.reserve(n_nodes);
+            if (precision == MPA_FP32) g.scn.reserve(n_nodes);
             for (int i = 0; i < n; ++i) {
                 Link& k = b->links[(size_t)g.links[(size_t)i]];
                 k.node_base = g.nodes.size();
@@ -303,6 +306,8 @@ int mpa_batch_create(const mpa_link* links, int32_t n_links, double L_km, int32_
                         c.post = sig * dz / c.pre;
                         g.nodes.push_back(c);
                     }
+                    if (precision == MPA_FP32)
+                        scan_nodes(k.map, u0, L_km, M, k.T, g.nodes.data() + g.nodes.size() - (size_t)(M + 1), &g.scn);
                 }
                 g.n_int = std::max(g.n_int, k.n_int);
             }
@@ -334,6 +339,8 @@ int mpa_batch_create(const mpa_link* links, int32_t n_links, double L_km, int32_
             if (precision == MPA_FP32) off = align256(off + (size_t)n * N * sizeof(float2));
             g.off_nodes = off;
             off = align256(off + g.nodes.size() * sizeof(NodeC));
+            g.off_scn = off;
+            off = align256(off + g.scn.size() * sizeof(ScanNode));
             g.off_loff = off;
             off = align256(off + g.loff.size() * sizeof(int));
             g.off_gain = off;
@@ -383,6 +390,8 @@ int mpa_batch_set_workspace(mpa_batch* b, void* ws, size_t bytes) {
     for (auto& g : b->groups) {
         MPA_TRY(cudaMemcpy(b->ws + g.off_nodes, g.nodes.data(), g.nodes.size() * sizeof(NodeC),
                            cudaMemcpyHostToDevice));
+        if (!g.scn.empty())
+            MPA_TRY(cudaMemcpy(b->ws + g.off_scn, g.scn.data(), g.scn.size() * sizeof(ScanNode), cudaMemcpyHostToDevice));
         MPA_TRY(cudaMemcpy(b->ws + g.off_loff, g.loff.data(), g.loff.size() * sizeof(int), cudaMemcpyHostToDevice));
         MPA_TRY(cudaMemcpy(b->ws + g.off_gain, g.gain.data(), g.gain.size() * sizeof(double), cudaMemcpyHostToDevice));
         MPA_TRY(cudaMemset(b->ws + g.off_err, 0, sizeof(unsigned int)));
@@ -527,6 +536,7 @@ int mpa_batch_autotune(mpa_batch* b, mpa_stream stream) {
                                              reinterpret_cast<float2*>(b->ws + g.off_psi0c),
                                              reinterpret_cast<double2*>(b->ws + g.off_state),
                                              reinterpret_cast<const NodeC*>(b->ws + g.off_nodes),
+                                             reinterpret_cast<const ScanNode*>(b->ws + g.off_scn),
                                              reinterpret_cast<const int*>(b->ws + g.off_loff),
                                              reinterpret_cast<const double*>(b->ws + g.off_gain),
                                              group_monitor(b->ws, b->ws_bytes, g, b->spin_limit), 1, nullptr, st)
@@ -535,6 +545,7 @@ int mpa_batch_autotune(mpa_batch* b, mpa_stream stream) {
                                               reinterpret_cast<double2*>(b->ws + g.off_psi0c),
                                               reinterpret_cast<double2*>(b->ws + g.off_state),
                                               reinterpret_cast<const NodeC*>(b->ws + g.off_nodes),
+                                              reinterpret_cast<const ScanNode*>(b->ws + g.off_scn),
                                               reinterpret_cast<const int*>(b->ws + g.off_loff),
                                               reinterpret_cast<const double*>(b->ws + g.off_gain),
                                               group_monitor(b->ws, b->ws_bytes, g, b->spin_limit), 1, nullptr, st);

@@ -214,18 +214,34 @@ struct NodeC {
     double post; // MPA: sigma(z_j) dz / pre (weight of V_j in Eq. (6))
 };
 
+// The scan's per-node constants (FP32): the step of the phase coefficients
+// from node j to node j + 1 (the phases of Eq. (6) are walked node by node,
+// theta_{j+1} = theta_j + k'^2 da + k'^3 db), the real factors of NodeC in
+// FP32, twice each (the operands of packed products), and the next node
+// whose step differs from this one's (INT_MAX: none; the step is the same for
+// all nodes of one fiber segment).
+struct ScanNode {
+    unsigned long long da_hi, da_lo, db_hi, db_lo;
+    float pre[2], post[2];
+    int next, pad[3];
+};
+
 // frac(k'^2 a + k'^3 b) as an unsigned Q0.64 number of turns (within 2 ulp).
 // frac(k'^3 b) = frac(k' frac(k'^2 b)) since k'^3 b - k' frac(k'^2 b) is an
 // integer multiple of k'.
-__device__ __forceinline__ unsigned long long phase_q64(long long kp, const NodeC& c) {
+__device__ __forceinline__ unsigned long long phase_q64(long long kp, unsigned long long a_hi, unsigned long long a_lo,
+                                                        unsigned long long b_hi, unsigned long long b_lo) {
     const unsigned long long ak = (unsigned long long)(kp < 0 ? -kp : kp);
     const unsigned long long u = ak * ak;  // < 2^50 for N <= 2^25
-    const unsigned long long ta = u * c.a_hi + __umul64hi(u, c.a_lo);
-    const unsigned long long f_lo = u * c.b_lo;
-    const unsigned long long f_hi = u * c.b_hi + __umul64hi(u, c.b_lo);
+    const unsigned long long ta = u * a_hi + __umul64hi(u, a_lo);
+    const unsigned long long f_lo = u * b_lo;
+    const unsigned long long f_hi = u * b_hi + __umul64hi(u, b_lo);
     unsigned long long tb = ak * f_hi + __umul64hi(ak, f_lo);
     if (kp < 0) tb = 0ull - tb;  // odd power of k'
     return ta + tb;
+}
+__device__ __forceinline__ unsigned long long phase_q64(long long kp, const NodeC& c) {
+    return phase_q64(kp, c.a_hi, c.a_lo, c.b_hi, c.b_lo);
 }
 
 // exp(2 pi i theta) for theta a Q0.64 fraction of a turn: reinterpret as a
@@ -279,6 +295,32 @@ __device__ __forceinline__ float2 expi_turns_poly(unsigned long long th) {
     const unsigned neg = (unsigned)(q & 2) << 30;
     return make_float2(__uint_as_float(__float_as_uint(a) ^ neg), __uint_as_float(__float_as_uint(b) ^ neg));
 }
+
+#if MPA_F32X2
+// expi_turns_poly of two phases at once: the same operations, the series of
+// both phases in the two lanes of packed instructions, and the quarter turn
+// taken from the bits of theta + 1/8 turn (bit 31 of its high word: half a
+// turn on, a sign; bit 30: a quarter turn on, cos and sin swapped).
+__device__ __forceinline__ void expi_turns_poly2(unsigned long long ta, unsigned long long tb, float2& ea, float2& eb) {
+    const unsigned ha = (unsigned)(ta >> 32) + (1u << 29), hb = (unsigned)(tb >> 32) + (1u << 29);
+    const int da = (int)(ha & 0x3FFFFFFFu) - (1 << 29), db = (int)(hb & 0x3FFFFFFFu) - (1 << 29);
+    const float2 k = make_float2(1.4629180792671596e-09f, 1.4629180792671596e-09f);  // 2 pi 2^-32
+    const float2 x = mul2(make_float2(__int2float_rn(da), __int2float_rn(db)), k), x2 = mul2(x, x);
+    float2 c = fma2(x2, make_float2(2.4801587e-05f, 2.4801587e-05f), make_float2(-1.3888889e-03f, -1.3888889e-03f));
+    c = fma2(c, x2, make_float2(4.1666668e-02f, 4.1666668e-02f));
+    c = fma2(c, x2, make_float2(-0.5f, -0.5f));
+    c = fma2(c, x2, make_float2(1.0f, 1.0f));
+    float2 sn = fma2(x2, make_float2(2.7557319e-06f, 2.7557319e-06f), make_float2(-1.9841270e-04f, -1.9841270e-04f));
+    sn = fma2(sn, x2, make_float2(8.3333338e-03f, 8.3333338e-03f));
+    sn = fma2(sn, x2, make_float2(-0.16666667f, -0.16666667f));
+    sn = fma2(mul2(sn, x2), x, x);
+    const bool oa = (ha & 0x40000000u) != 0, ob = (hb & 0x40000000u) != 0;
+    const unsigned na = ha & 0x80000000u, nb = hb & 0x80000000u;
+    const float ax = oa ? -sn.x : c.x, ay = oa ? c.x : sn.x, bx = ob ? -sn.y : c.y, by = ob ? c.y : sn.y;
+    ea = make_float2(__uint_as_float(__float_as_uint(ax) ^ na), __uint_as_float(__float_as_uint(ay) ^ na));
+    eb = make_float2(__uint_as_float(__float_as_uint(bx) ^ nb), __uint_as_float(__float_as_uint(by) ^ nb));
+}
+#endif
 
 // (sin, cos) of a Kerr phase phi = sigma |A|^2 dz of the split-step.  These
 // phases are small (about 1e-3 rad on the benchmark links), so for

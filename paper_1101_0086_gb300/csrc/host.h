@@ -294,8 +294,11 @@ inline int fft_inverse(const Split& s, cx<T>* spec, cx<T>* out, cudaStream_t st)
 // the layout cannot work in place).
 template <typename T>
 int mpa_levels(const Split& s, int M, int n_iter, int nl, cx<T>* psi, cx<T>* work, cx<T>* psi0c, double2* state,
-               const NodeC* nodes, const int* loff, const double* gain, const Monitor& mon, int scan_mode,
-               double2* out, cudaStream_t st);
+               const NodeC* nodes, const ScanNode* scn, const int* loff, const double* gain, const Monitor& mon,
+               int scan_mode, double2* out, cudaStream_t st);
+// The scan's constants of the interval that starts at u0 within the period
+// (M + 1 entries appended), nodes[0..M] being its node constants.
+void scan_nodes(const HostMap& m, double u0, double L, int M, double T, const NodeC* nodes, std::vector<ScanNode>* out);
 // Whether a plan or batch group of N modes in this precision gets the
 // second set of node buffers (the staged column passes need N1 >= 32).
 inline bool wants_work_buffers(long long N, int prec) { return prec == MPA_FP32 && N >= (1ll << 13); }

@@ -36,7 +36,7 @@ static cudaError_t kcs_one(const KCParams<float>& p, cudaStream_t st) {
     if (prof) {
         const double cs = (double)sizeof(cx<float>), tile = (double)p.ncols * L;
         const double rd = p.src_stride == 0 ? (double)p.ncols / p.npl * L : tile;
-        prof_end(prof_kc_kind(MODE), st, (rd + tile) * cs);
+        prof_end(prof_kc_kind(MODE, p.err != nullptr), st, (rd + tile) * cs);
     }
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError();
@@ -49,7 +49,7 @@ template <int L> static bool kcs_fits(const KCParams<float>& p) {
 }
 
 bool kc_staged(int mode, int logL, const KCParams<float>& p) {
-    if (!MPA_KC_STAGED || !p.err || (mode != KC_MPA_PRE && mode != KC_MPA_POST) || p.npl <= 0) return false;
+    if (!MPA_KC_STAGED || !p.err || mode == KC_SS_STEP || mode == KC_MPA_POST || p.npl <= 0) return false;
     switch (logL) {
         case 8: return kcs_fits<256>(p);
         case 9: return kcs_fits<512>(p);
@@ -70,7 +70,12 @@ int kcs_tile_log_cols(int logL) {
 }
 
 template <int L> static cudaError_t kcs_mode(int mode, const KCParams<float>& p, cudaStream_t st) {
-    return mode == KC_MPA_PRE ? kcs_one<L, KC_MPA_PRE>(p, st) : kcs_one<L, KC_MPA_POST>(p, st);
+    switch (mode) {
+        case KC_MPA_PRE: return kcs_one<L, KC_MPA_PRE>(p, st);
+        case KC_INV: return kcs_one<L, KC_INV>(p, st);
+        case KC_FWD: return kcs_one<L, KC_FWD>(p, st);
+    }
+    return cudaErrorInvalidValue;
 }
 
 template <int L, int MODE>
@@ -100,7 +105,7 @@ static cudaError_t kc_one(const KCParams<float>& pin, cudaStream_t st) {
         // (a shared source, src_stride == 0, is read once for all nodes)
         const double cs = (double)sizeof(cx<float>), tile = (double)p.ncols * L;
         const double rd = p.src_stride == 0 ? (double)p.ncols / p.npl * L : tile;
-        prof_end(prof_kc_kind(MODE), st, (rd + tile) * cs);
+        prof_end(prof_kc_kind(MODE, p.err != nullptr), st, (rd + tile) * cs);
     }
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError();

@@ -30,7 +30,7 @@ static cudaError_t kc_one(const KCParams<double>& pin, cudaStream_t st) {
         // (a shared source, src_stride == 0, is read once for all nodes)
         const double cs = (double)sizeof(cx<double>), tile = (double)p.ncols * L;
         const double rd = p.src_stride == 0 ? (double)p.ncols / p.npl * L : tile;
-        prof_end(prof_kc_kind(MODE), st, (rd + tile) * cs);
+        prof_end(prof_kc_kind(MODE, p.err != nullptr), st, (rd + tile) * cs);
     }
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError();

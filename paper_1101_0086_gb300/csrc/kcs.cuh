@@ -1,7 +1,7 @@
 // Staged, persistent column pass (FP32; the MPA column passes): the
 // arithmetic of kc_kernel in modes KC_MPA_PRE (phase exp(i beta_j + int G),
-// inverse column DFTs, outer factor W_N^{-n2 k1}) and KC_MPA_POST (forward
-// column DFTs, V_j of Eq. (6)) on the schedule of the staged row pass
+// inverse column DFTs, outer factor W_N^{-n2 k1}), KC_INV (the same without
+// the phase) and KC_FWD (forward column DFTs) on the schedule of the staged row pass
 // (krs.cuh): one CTA per SM, two groups of NT threads taking the CTA's
 // tiles in turn, and one staging buffer that the next tile streams into
 // while the current ones are transformed.
@@ -81,10 +81,6 @@ __host__ __device__ __forceinline__ float2* kcs_dst(const KCParams<float>& p, in
     return p.tiled_out ? b + c * L : b + c;
 }
 
-// 16-byte global -> shared copy through L2 (cp.async.cg)
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-}
 // barrier b receives one arrival from this thread once all of its earlier
 // cp.async copies have landed (the arrival is counted in b's expected count)
 __device__ __forceinline__ void cp_async_arrive(unsigned long long* b) {
@@ -93,10 +89,10 @@ __device__ __forceinline__ void cp_async_arrive(unsigned long long* b) {
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Group-wide: the NT threads start the copies of tile t (L row segments of
-// G elements) into the stage, and three of them the copy of the tile's node
-// constants into `slot`; each thread arrives on barrier b when its copies
+// G elements) into the stage, and (NODES) three of them the copy of the
+// tile's node constants into `slot`; each thread arrives on barrier b when its copies
 // have landed.
-template <int L>
+template <int L, bool NODES>
 __device__ __forceinline__ void kcs_fetch(const KCParams<float>& p, int t, float2* stage, NodeC* slot,
                                           unsigned long long* b, int tid) {
     constexpr int G = KCSTile<L>::G, NT = KCSTile<L>::NT;
@@ -114,7 +110,7 @@ __device__ __forceinline__ void kcs_fetch(const KCParams<float>& p, int t, float
         const char* from = src + (long long)row * rs * (long long)sizeof(float2) + ch * 16;
         if (MPA_DBG_OK(p.dbg, from, 16)) cp_async16(dst + (size_t)row * G * sizeof(float2) + ch * 16, from);
     }
-    if (tid < (int)(sizeof(NodeC) / 16) && MPA_DBG_OK(p.dbg, p.loff + l, sizeof(int))) {
+    if (NODES && tid < (int)(sizeof(NodeC) / 16) && MPA_DBG_OK(p.dbg, p.loff + l, sizeof(int))) {
         const char* from = reinterpret_cast<const char*>(p.nodes + p.loff[l] + jn) + 16 * tid;
         if (MPA_DBG_OK(p.dbg, from, 16)) cp_async16(reinterpret_cast<char*>(slot) + 16 * tid, from);
     }
@@ -144,13 +140,13 @@ __device__ __forceinline__ void kcs_prefetch(const KCParams<float>& p, int t, in
 template <int L, int MODE>
 __global__ void __launch_bounds__(KCSGeom<L>::THREADS, 1)
     kcs_kernel(const KCParams<float> p) {
-    static_assert(MODE == KC_MPA_PRE || MODE == KC_MPA_POST, "the MPA column passes");
+    static_assert(MODE == KC_MPA_PRE || MODE == KC_INV || MODE == KC_FWD, "the MPA column passes");
     typedef float2 C;
     typedef KCSTile<L> Gm;
     typedef KCSGeom<L> SG;
     typedef Tiling<float> P;
     constexpr int G = Gm::G, NT = Gm::NT;
-    constexpr bool INV = MODE == KC_MPA_PRE;
+    constexpr bool INV = MODE != KC_FWD, PRE = MODE == KC_MPA_PRE;
     typedef Xform<float, L, G, NT, P::RMAX, +1, LAYOUT_COL, P::PSH, true, 1> XF;
     typedef Xform<float, L, G, NT, P::RMAX, -1, LAYOUT_COL, P::PSH, false, 1> XI;
     typedef typename std::conditional<INV, XI, XF>::type XA;
@@ -175,7 +171,7 @@ __global__ void __launch_bounds__(KCSGeom<L>::THREADS, 1)
     tw_init<float, L>(thi, tlo, (int)threadIdx.x, SG::THREADS);
     __syncthreads();
     // the first tile is copied by group 1 (whose own first tile comes later)
-    if (grp == 1 && (int)blockIdx.x < ntiles) kcs_fetch<L>(p, blockIdx.x, stage, &nslot[0], &bar[0], tid);
+    if (grp == 1 && (int)blockIdx.x < ntiles) kcs_fetch<L, PRE>(p, blockIdx.x, stage, &nslot[0], &bar[0], tid);
 
     unsigned k = 0;
     for (int i = grp;; i += 2, ++k) {
@@ -205,7 +201,7 @@ __global__ void __launch_bounds__(KCSGeom<L>::THREADS, 1)
         for (int q = 0; q < XA::Q0; ++q) {
             int j, g;
             bmap<LAYOUT_COL, L, G, XA::R0>(tid + q * NT, j, g);
-            if constexpr (INV) {
+            if constexpr (PRE) {
                 const long long c = tc0 + g;
                 const NodeC nc = nslot[i & 3];  // copied with the tile
                 // phases in the order of their finite differences: s = -R0/2 .. R0/2-1,
@@ -240,7 +236,7 @@ __global__ void __launch_bounds__(KCSGeom<L>::THREADS, 1)
         constexpr bool LATE = INV && (L == 256 || L == 2048);
         auto fetch_next = [&] {
             const int tn = t + (int)gridDim.x;
-            if (tn < ntiles) kcs_fetch<L>(p, tn, stage, &nslot[(i + 1) & 3], &bar[grp ^ 1], tid);
+            if (tn < ntiles) kcs_fetch<L, PRE>(p, tn, stage, &nslot[(i + 1) & 3], &bar[grp ^ 1], tid);
             constexpr bool PF = (MPA_KCS_L2PF >> (INV ? 0 : 1)) & 1;
             if constexpr (PF) {
                 const int tp = tn + (int)gridDim.x;
@@ -259,7 +255,6 @@ __global__ void __launch_bounds__(KCSGeom<L>::THREADS, 1)
         for (int q = 0; q < QO; ++q) {
             int j, g;
             bmap<LAYOUT_COL, L, G, RO>(tid + q * NT, j, g);
-            const long long c = tc0 + g;
             long long rs;
             // natural order, or the tile layout: the tile block at column tc0, element g
             C* dst = kcs_dst<L, G>(p, tl, tjn, tc0, rs) + g;
@@ -276,16 +271,10 @@ __global__ void __launch_bounds__(KCSGeom<L>::THREADS, 1)
                     if (MPA_DBG_OK(p.dbg, dst + (long long)row * rs, sizeof(C))) dst[(long long)row * rs] = cmul(vout[q][r], w);
                 }
             } else {
-                const NodeC nc = nslot[i & 3];  // copied with the tile
-                const long long D = (long long)p.N1 * (L / RO);
-                PhaseRun pr(c + (long long)j * p.N1 - (long long)(RO / 2) * D, D, nc);
 #pragma unroll
-                for (int u = 0; u < RO; ++u) {
-                    const int r = (u + RO / 2) % RO;
+                for (int r = 0; r < RO; ++r) {
                     const int row = j + r * (L / RO);
-                    // V_j = sigma(z_j) dz F[|A_j|^2 A_j] exp(-i beta(w, z_j) - int G)   (Eq. (6))
-                    const C v = cscale(cmul(vout[q][r], cconj(expi_turns_poly(pr.next()))), (float)nc.post);
-                    if (MPA_DBG_OK(p.dbg, dst + (long long)row * rs, sizeof(C))) dst[(long long)row * rs] = v;
+                    if (MPA_DBG_OK(p.dbg, dst + (long long)row * rs, sizeof(C))) dst[(long long)row * rs] = vout[q][r];
                 }
             }
         }

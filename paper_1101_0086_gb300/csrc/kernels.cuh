@@ -22,6 +22,7 @@
 //                     every frequency, fused with step 7 on the last iteration.
 #pragma once
 
+#include <climits>
 #include <type_traits>
 
 #include "device.cuh"
@@ -485,9 +486,11 @@ __global__ void __launch_bounds__(KRGeom<T, L>::NT, KRGeom<T, L>::NT <= 256 ? MP
 // N small enough that one spectrum fits in a CTA's shared memory (N <= 2^14
 // FP32, 2^13 FP64): G = TE/N nodes per CTA, each a row of the row-pass tile
 // layout holding its spectrum in natural order:
-//   A_hat = psi_j exp(i beta_j + int G)        (phase at the load, step 2)
+//   A_hat = psi_j exp(i beta_j + int G)        (phase at the load, step 2; PIN)
 //   A = F^-1[A_hat]; U = |A|^2 A; F[U]          (steps 3-4, in shared memory)
-//   V_j = F[U] sigma_j dz exp(-i beta_j - int G)   (at the store, Eq. (6))
+//   V_j = F[U] sigma_j dz exp(-i beta_j - int G)   (at the store, Eq. (6); POUT)
+// Without PIN the source holds A_hat_j already, without POUT the destination
+// receives F[U] (ScanParams::phases: the scan applies the phases).
 // One HBM (or L2) round trip per node instead of the three of the column,
 // row and column passes, no four-step outer factors.  Node addressing as in
 // KCParams (nl links x npl nodes, psi_0 shared by node 0).
@@ -503,6 +506,7 @@ template <typename T> struct KNParams {
     const NodeC* nodes;  // link l, node jn at nodes[loff[l] + jn]
     const int* loff;
     T inv_n;
+    bool phase_in, phase_out;  // kn_launch: the phases applied at the load and at the store
     DbgRange dbg;  // checked range of the debug build
 };
 
@@ -516,7 +520,7 @@ template <typename T, int L> struct KNGeom {
 
 // The node rows row0 .. row0 + G - 1 of a launch (one tile) through steps
 // 2-4 and the weight of Eq. (6); the block's threads and shared memory.
-template <typename T, int L, bool CG>
+template <typename T, int L, bool CG, bool PIN, bool POUT>
 __device__ __forceinline__ void kn_tile(const KNParams<T>& p, long long row0, unsigned char* smem_raw) {
     typedef cx<T> C;
     typedef KNGeom<T, L> Gm;
@@ -545,6 +549,14 @@ __device__ __forceinline__ void kn_tile(const KNParams<T>& p, long long row0, un
         const int node = ok ? (int)row : 0;
         const int l = node / p.npl, jn = node - l * p.npl;
         const C* src = (p.src0 && jn == 0) ? p.src0 + l * p.src0_lstride : p.src + l * p.src_lstride + jn * p.src_stride;
+        if constexpr (!PIN) {
+#pragma unroll
+            for (int r = 0; r < XI::R0; ++r) {
+                const int k = j + r * (L / XI::R0);
+                vin[q][r] = ok && MPA_DBG_OK(p.dbg, src + k, sizeof(C)) ? ldx<CG>(src + k) : mkc(T(0), T(0));
+            }
+            continue;
+        }
         NodeC nc{};
         if (MPA_DBG_OK(p.dbg, p.loff + l, sizeof(int)) && MPA_DBG_OK(p.dbg, p.nodes + p.loff[l] + jn, sizeof(NodeC)))
             nc = p.nodes[p.loff[l] + jn];
@@ -585,6 +597,14 @@ __device__ __forceinline__ void kn_tile(const KNParams<T>& p, long long row0, un
         const int node = (int)row;
         const int l = node / p.npl, jn = node - l * p.npl;
         C* dst = p.dst + l * p.dst_lstride + jn * p.dst_stride;
+        if constexpr (!POUT) {
+#pragma unroll
+            for (int r = 0; r < XF::RL; ++r) {
+                const int k = j + r * (L / XF::RL);
+                if (MPA_DBG_OK(p.dbg, dst + k, sizeof(C))) dst[k] = vout[q][r];
+            }
+            continue;
+        }
         NodeC nc{};
         if (MPA_DBG_OK(p.dbg, p.loff + l, sizeof(int)) && MPA_DBG_OK(p.dbg, p.nodes + p.loff[l] + jn, sizeof(NodeC)))
             nc = p.nodes[p.loff[l] + jn];
@@ -601,11 +621,11 @@ __device__ __forceinline__ void kn_tile(const KNParams<T>& p, long long row0, un
     }
 }
 
-template <typename T, int L>
+template <typename T, int L, bool PIN, bool POUT>
 __global__ void __launch_bounds__(KNGeom<T, L>::NT, KNGeom<T, L>::NT <= 256 ? MPA_KR_MINB : 1)
     kn_kernel(const KNParams<T> p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    kn_tile<T, L, false>(p, (long long)blockIdx.x * KNGeom<T, L>::G, smem_raw);
+    kn_tile<T, L, false, PIN, POUT>(p, (long long)blockIdx.x * KNGeom<T, L>::G, smem_raw);
 }
 
 // ------------------------------------------------------------------
@@ -846,7 +866,10 @@ __global__ void __launch_bounds__(KCWGeom<L>::NT, KCWGeom<L>::NT <= 256 ? MPA_KC
 //   psi^{(n+1)}_l = psi_0 + i (V_0/2 + sum_{j=1}^{l-1} V_j + V_l/2),
 // with V_j stored in psi[j] (node 0 holds V_0).  FP32 sums are Kahan-
 // compensated; the final value at node M is formed in FP64.
-//   mode 0: write psi^{(n+1)}_j into psi[j] (next iteration)
+//   mode 0: write psi^{(n+1)}_j into psi[j], j >= 1 (next iteration)
+// With `phases`, psi[j] holds F_j = F[|A_j|^2 A_j] instead, the scan forms
+// V_j = sigma_j dz F_j exp(-i beta_j - int G) itself, and mode 0 writes
+// A_hat^{(n+1)}_j = psi^{(n+1)}_j exp(i beta_j + int G).
 //   mode 1: step 7: state <- psi_M exp(i beta(w, z0+L) + int G) * gain, psi0c <- state
 //   mode 2: out <- psi_M (FP64, no step 7)
 //
@@ -898,7 +921,9 @@ template <typename T> struct ScanParams {
     cx<T>* psi0c_out;    // mode 1: working-precision copy of the new state
     double2* out;        // mode 2
     int mode;
-    const NodeC* nodes;  // node M of link l: nodes[loff[l] + M]
+    const NodeC* nodes;  // node j of link l: nodes[loff[l] + j]
+    const ScanNode* scn; // phases, FP32: the scan's constants, indexed as nodes
+    bool phases;         // psi holds F_j and receives A_hat_j (the scan applies the phases)
     const int* loff;
     const double* gain;  // amplifier gain at the interval end, per link
     unsigned int* err;
@@ -964,53 +989,49 @@ __device__ __forceinline__ void conv_close(ConvState* cs, unsigned int* err, dou
     }
 }
 
-// 8-byte global -> shared copy (cp.async.ca) and its commit / wait groups
-__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait_group() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
 // What follows the sums at one frequency (position i, natural index k) of
-// link l, D = (sx, sy) being the trapezoid sum of Eq. (6) at node M: the
-// Picard increment check, and at the last level step 7 (mode 1) or psi_M
-// (mode 2).  BLOCK: every thread of the block calls, and the check's sums go
-// through a block reduction; else one whole warp of the block calls, and its
-// sums are the block's.
-template <typename T, bool CG, bool BLOCK>
-__device__ __forceinline__ void scan_node_m(const ScanParams<T>& p, int l, long long i, long long k, cx<T> p0, double sx,
-                                            double sy, unsigned nblk) {
+// link l, D = (sx, sy) being the trapezoid sum of Eq. (6) at node M.
+// The frequency's terms of the Picard increment check (D is kept for the
+// next level):
+template <typename T, bool CG>
+__device__ __forceinline__ void scan_increment(const ScanParams<T>& p, int l, long long i, cx<T> p0, double sx, double sy,
+                                               double& d2, double& p2) {
+    const long long lo = (long long)l * p.N;
+    // Picard increment at node M against the previous level's D
+    double dx = sx, dy = sy;
+    if (p.level > 0) {
+        const float2 d0 = MPA_DBG_OK(p.dbg, p.dprev + lo + i, sizeof(float2)) ? ldx<CG>(p.dprev + lo + i)
+                                                                             : make_float2(0.f, 0.f);
+        dx -= (double)d0.x;
+        dy -= (double)d0.y;
+    }
+    if (p.level < p.n_iter - 1 && MPA_DBG_OK(p.dbg, p.dprev + lo + i, sizeof(float2)))
+        p.dprev[lo + i] = make_float2((float)sx, (float)sy);
+    const double px = (double)p0.x - sy, py = (double)p0.y + sx;
+    d2 += dx * dx + dy * dy;
+    p2 += px * px + py * py;
+}
+// The check's sums of a block.  BLOCK: every thread of the block calls, the
+// sums go through a block reduction; else one whole warp of the block calls,
+// and its sums are the block's.
+template <typename T, bool BLOCK>
+__device__ __forceinline__ void scan_check(const ScanParams<T>& p, int l, double d2, double p2, unsigned nblk) {
+    if constexpr (BLOCK) {
+        conv_close(p.conv + l, p.err, d2, p2, p.level, p.n_iter - 1, p.floor_rel, nblk);
+    } else {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            d2 += __shfl_xor_sync(0xffffffffu, d2, o);
+            p2 += __shfl_xor_sync(0xffffffffu, p2, o);
+        }
+        if ((threadIdx.x & 31) == 0) conv_level(p.conv + l, p.err, d2, p2, p.level, p.n_iter - 1, p.floor_rel, nblk);
+    }
+}
+// At the last level, step 7 (mode 1) or psi_M (mode 2):
+template <typename T, bool CG>
+__device__ __forceinline__ void scan_finish(const ScanParams<T>& p, int l, long long k, double sx, double sy) {
     typedef cx<T> C;
     const long long lo = (long long)l * p.N;
-    if (p.conv) {
-        // Picard increment at node M against the previous level's D
-        double dx = sx, dy = sy;
-        if (p.level > 0) {
-            const float2 d0 = MPA_DBG_OK(p.dbg, p.dprev + lo + i, sizeof(float2)) ? ldx<CG>(p.dprev + lo + i)
-                                                                                 : make_float2(0.f, 0.f);
-            dx -= (double)d0.x;
-            dy -= (double)d0.y;
-        }
-        if (p.level < p.n_iter - 1 && MPA_DBG_OK(p.dbg, p.dprev + lo + i, sizeof(float2)))
-            p.dprev[lo + i] = make_float2((float)sx, (float)sy);
-        const double px = (double)p0.x - sy, py = (double)p0.y + sx;
-        double d2 = dx * dx + dy * dy, p2 = px * px + py * py;
-        if constexpr (BLOCK) {
-            conv_close(p.conv + l, p.err, d2, p2, p.level, p.n_iter - 1, p.floor_rel, nblk);
-        } else {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                d2 += __shfl_xor_sync(0xffffffffu, d2, o);
-                p2 += __shfl_xor_sync(0xffffffffu, p2, o);
-            }
-            if ((threadIdx.x & 31) == 0)
-                conv_level(p.conv + l, p.err, d2, p2, p.level, p.n_iter - 1, p.floor_rel, nblk);
-        }
-    }
-    if (p.mode == 0) return;
     const double2 s0 = MPA_DBG_OK(p.dbg, p.state + lo + k, sizeof(double2)) ? ldx<CG>(p.state + lo + k)
                                                                           : make_double2(0.0, 0.0);
     const double2 psiM = make_double2(s0.x - sy, s0.y + sx);
@@ -1030,113 +1051,269 @@ __device__ __forceinline__ void scan_node_m(const ScanParams<T>& p, int l, long 
     if (!(isfinite(a.x) && isfinite(a.y))) atomicOr(p.err, ERR_NONFINITE);
 }
 
+// All of it for one frequency, and for the pair k, k + 1 at positions i, i + 1.
+template <typename T, bool CG, bool BLOCK>
+__device__ __forceinline__ void scan_node_m(const ScanParams<T>& p, int l, long long i, long long k, cx<T> p0, double sx,
+                                            double sy, unsigned nblk) {
+    if (p.conv) {
+        double d2 = 0.0, p2 = 0.0;
+        scan_increment<T, CG>(p, l, i, p0, sx, sy, d2, p2);
+        scan_check<T, BLOCK>(p, l, d2, p2, nblk);
+    }
+    if (p.mode != 0) scan_finish<T, CG>(p, l, k, sx, sy);
+}
+template <bool BLOCK>
+__device__ __forceinline__ void scan_pair_m(const ScanParams<float>& p, int l, long long i, long long k, float2 pa, float2 pb,
+                                            double ax, double ay, double bx, double by, unsigned nblk) {
+    if (p.conv) {
+        double d2 = 0.0, p2 = 0.0;
+        scan_increment<float, false>(p, l, i, pa, ax, ay, d2, p2);
+        scan_increment<float, false>(p, l, i + 1, pb, bx, by, d2, p2);
+        scan_check<float, BLOCK>(p, l, d2, p2, nblk);
+    }
+    if (p.mode != 0) {
+        scan_finish<float, false>(p, l, k, ax, ay);
+        scan_finish<float, false>(p, l, k + 1, bx, by);
+    }
+}
+
+// s += v, Kahan-compensated in FP32 (c carries the lost low-order part; the
+// float2 sums and differences are packed instructions), plain in FP64.
+template <class C> __device__ __forceinline__ void scan_add(C& s, C& c, C v) {
+    if constexpr (sizeof(C) == 8) {
+        const C y = csub(v, c), t = cadd(s, y);
+        c = csub(csub(t, s), y);
+        s = t;
+    } else {
+        s = cadd(s, v);
+    }
+}
+// s - c + v / 2
+template <class C> __device__ __forceinline__ C scan_half(C s, C c, C v) {
+    if constexpr (sizeof(C) == 8) return cadd(csub(s, c), cscale(v, 0.5f));
+    else return mkc(s.x + 0.5 * v.x, s.y + 0.5 * v.y);
+}
+
+// 16-byte global -> shared copy through L2 (cp.async.cg) and its commit /
+// wait groups
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait_group() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // Frequency k of link l (one thread each; a block of consecutive
 // frequencies, nblk blocks per link).  N is a multiple of the block size (a
 // power of two >= 256), so every thread has a frequency and takes part in
 // the block reduction of the increment check.
-// S > 0 (FP32 only): the thread's V_j travel S nodes ahead through its own S
-// shared-memory slots (ring[slot * blockDim.x + threadIdx.x]) by 8-byte
-// cp.async, one commit group per node, so the bytes in flight do not cost
-// registers; S = 0 keeps U = 8 nodes ahead in registers.
-template <typename T, bool CG, int S = 0>
-__device__ __forceinline__ void scan_freq(const ScanParams<T>& p, int l, long long i, unsigned nblk,
-                                          cx<T>* ring = nullptr) {
+// PH (ScanParams::phases; FP64 plans): psi holds F_j and receives A_hat_j,
+// every phase from its node's own constants; else (also the persistent batch
+// kernel) it holds V_j and receives psi_j.  Nodes are loaded 8 ahead.
+template <typename T, bool CG, bool PH>
+__device__ __forceinline__ void scan_freq(const ScanParams<T>& p, int l, long long i, unsigned nblk) {
     typedef cx<T> C;
-    static_assert(S == 0 || sizeof(T) == 4, "staged node reads of complex64");
     const long long lo = (long long)l * p.N;
-    cx<T>* psi = p.psi + lo * (p.M + 1);
     // i: position in the node buffers; k: the frequency there (natural order)
+    cx<T>* psi = p.psi + lo * (p.M + 1) + i;
     const long long k = p.tile_logG > 0 ? tile_to_natural(i, p.tile_logG, p.tile_logL, p.N) : i;
+    const long long kk = signed_k(k, p.N);
     const C zero = mkc(T(0), T(0));
-    const C v0 = MPA_DBG_OK(p.dbg, psi + i, sizeof(C)) ? ldx<CG>(psi + i) : zero;
-    T rx = T(0.5) * v0.x, ry = T(0.5) * v0.y, cxx = T(0), cyy = T(0);
+    const C v0 = MPA_DBG_OK(p.dbg, psi, sizeof(C)) ? ldx<CG>(psi) : zero;
     const C p0 = MPA_DBG_OK(p.dbg, p.psi0c + lo + k, sizeof(C)) ? ldx<CG>(p.psi0c + lo + k) : zero;
-    C vl = v0;
-    // node j: psi^{(n+1)}_j = psi_0 + i (R + V_j/2), then R += V_j (Kahan in FP32)
-    auto node = [&](int j) {
-        if (p.mode == 0) {
-            const T sx = (rx - cxx) + T(0.5) * vl.x, sy = (ry - cyy) + T(0.5) * vl.y;
-            if (MPA_DBG_OK(p.dbg, psi + (long long)j * p.N + i, sizeof(C))) psi[(long long)j * p.N + i] = mkc(p0.x - sy, p0.y + sx);
-        }
-        if constexpr (sizeof(T) == 4) {
-            kahan_add(rx, cxx, vl.x);
-            kahan_add(ry, cyy, vl.y);
-        } else {
-            rx += vl.x;
-            ry += vl.y;
-        }
+    const NodeC* nodes = nullptr;
+    auto consts = [&](int j) {
+        NodeC nc{};
+        if (MPA_DBG_OK(p.dbg, nodes + j, sizeof(NodeC))) nc = nodes[j];
+        return nc;
     };
-    if constexpr (S > 0) {
-        // the loads never touch a node the loop has written (they run ahead)
-        C* mine = ring + threadIdx.x;
-#pragma unroll
-        for (int u = 0; u < S; ++u) {
-            if (1 + u <= p.M && MPA_DBG_OK(p.dbg, psi + (long long)(1 + u) * p.N + i, sizeof(C)))
-                cp_async8(mine + u * blockDim.x, psi + (long long)(1 + u) * p.N + i);
-            cp_async_commit();
+    C vl = v0;
+    if constexpr (PH) {
+        if (MPA_DBG_OK(p.dbg, p.loff + l, sizeof(int))) nodes = p.nodes + p.loff[l];
+        vl = cscale(v0, (T)consts(0).post);  // phase 0 and factor 1: V_0 = sigma_0 dz F_0
+    }
+    C r = cscale(vl, T(0.5)), c = zero;
+    // node j: psi^{(n+1)}_j = psi_0 + i (R + V_j/2), then R += V_j
+    auto node = [&](int j, C v) {
+        C ph;
+        vl = v;
+        if constexpr (PH) {
+            const NodeC nc = consts(j);
+            ph = expi_turns<T>(phase_q64(kk, nc));
+            vl = cscale(cmul(v, cconj(ph)), (T)nc.post);
+            ph = cscale(ph, (T)nc.pre);
         }
-        for (int j = 1; j <= p.M; ++j) {
-            cp_async_wait_group<S - 1>();  // node j's copy has landed
-            C* slot = mine + ((j - 1) % S) * blockDim.x;
-            vl = *slot;
-            node(j);
-            // the slot's value is consumed (node() used it): refill it with node j + S
-            if (j + S <= p.M && MPA_DBG_OK(p.dbg, psi + (long long)(j + S) * p.N + i, sizeof(C)))
-                cp_async8(slot, psi + (long long)(j + S) * p.N + i);
-            cp_async_commit();
+        if (p.mode == 0) {
+            const C h = scan_half(r, c, vl);
+            C o = mkc(p0.x - h.y, p0.y + h.x);
+            if constexpr (PH) o = cmul(o, ph);
+            if (MPA_DBG_OK(p.dbg, psi + (long long)j * p.N, sizeof(C))) psi[(long long)j * p.N] = o;
         }
-        cp_async_wait_group<0>();
-    } else {
-        // V_j are loaded U nodes ahead of their use (more loads in flight per
-        // thread; the loads never touch a node the loop has written)
-        constexpr int U = 8;
-        C nxt[U];
+        scan_add(r, c, vl);
+    };
+    // the loads never touch a node the loop has written (they run ahead)
+    constexpr int U = 8;
+    C nxt[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-            nxt[u] = (1 + u <= p.M && MPA_DBG_OK(p.dbg, psi + (long long)(1 + u) * p.N + i, sizeof(C)))
-                         ? ldx<CG>(psi + (long long)(1 + u) * p.N + i)
+    for (int u = 0; u < U; ++u)
+        nxt[u] = (1 + u <= p.M && MPA_DBG_OK(p.dbg, psi + (long long)(1 + u) * p.N, sizeof(C)))
+                     ? ldx<CG>(psi + (long long)(1 + u) * p.N)
+                     : zero;
+    for (int jb = 1; jb <= p.M; jb += U) {
+        C cur[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            cur[u] = nxt[u];
+            const int jn = jb + U + u;
+            nxt[u] = (jn <= p.M && MPA_DBG_OK(p.dbg, psi + (long long)jn * p.N, sizeof(C)))
+                         ? ldx<CG>(psi + (long long)jn * p.N)
                          : zero;
-        for (int jb = 1; jb <= p.M; jb += U) {
-            C cur[U];
+        }
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                cur[u] = nxt[u];
-                const int jn = jb + U + u;
-                nxt[u] = (jn <= p.M && MPA_DBG_OK(p.dbg, psi + (long long)jn * p.N + i, sizeof(C)))
-                             ? ldx<CG>(psi + (long long)jn * p.N + i)
-                             : zero;
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int j = jb + u;
-                if (j > p.M) break;
-                vl = cur[u];
-                node(j);
-            }
+        for (int u = 0; u < U; ++u) {
+            const int j = jb + u;
+            if (j > p.M) break;
+            node(j, cur[u]);
         }
     }
     // D = R_M - V_M/2 at node M in FP64 (psi_M = psi_0 + i D)
-    const double sx = ((double)rx - (double)cxx) - 0.5 * (double)vl.x;
-    const double sy = ((double)ry - (double)cyy) - 0.5 * (double)vl.y;
+    const double sx = ((double)r.x - (double)c.x) - 0.5 * (double)vl.x;
+    const double sy = ((double)r.y - (double)c.y) - 0.5 * (double)vl.y;
     scan_node_m<T, CG, true>(p, l, i, k, p0, sx, sy, nblk);
 }
 
-// Nodes in flight per thread of the FP32 scan (shared-memory slots; 0: the
-// register form).  Measured on the 2^20 link (126 nodes): 8 slots 31.6 ms
-// per 100 km (6.07 TB/s), 16 slots 34.8 ms (fewer resident blocks), the
-// register form (8 nodes ahead) 34.0 ms.
-#ifndef MPA_SCAN_STAGES
-#define MPA_SCAN_STAGES 8
-#endif
-template <typename T>
-__global__ void __launch_bounds__(256) scan_kernel(const ScanParams<T> p) {
-    if constexpr (sizeof(T) == 4 && MPA_SCAN_STAGES > 0) {
-        __shared__ float2 ring[MPA_SCAN_STAGES * 256];
-        scan_freq<T, false, MPA_SCAN_STAGES>(p, blockIdx.y, (long long)blockIdx.x * blockDim.x + threadIdx.x, gridDim.x,
-                                             ring);
-    } else {
-        scan_freq<T, false>(p, blockIdx.y, (long long)blockIdx.x * blockDim.x + threadIdx.x, gridDim.x);
+template <typename T, bool PH> __global__ void __launch_bounds__(256) scan_kernel(const ScanParams<T> p) {
+    scan_freq<T, false, PH>(p, blockIdx.y, (long long)blockIdx.x * blockDim.x + threadIdx.x, gridDim.x);
+}
+
+// ---- FP32: two neighbouring frequencies a thread.
+// The phases at a pair of frequencies k, k + 1, walked in node order: one
+// evaluation of the pair a node (packed), the phases advanced by their steps
+// (64-bit adds; a step is evaluated again only where the fiber segment
+// changes).
+struct PairWalk {
+    const ScanNode* sn;
+    const DbgRange& dbg;
+    long long ka, kb;
+    unsigned long long ta = 0, tb = 0, da = 0, db = 0;
+    int fresh = 0;  // the next node whose step is not the current one
+    __device__ __forceinline__ PairWalk(const ScanParams<float>& p, int l, long long k)
+        : sn(p.scn + (MPA_DBG_OK(p.dbg, p.loff + l, sizeof(int)) ? p.loff[l] : 0)), dbg(p.dbg), ka(signed_k(k, p.N)),
+          kb(signed_k(k + 1, p.N)) {}
+    // the step from node j on
+    __device__ __forceinline__ void step(int j) {
+        fresh = INT_MAX;
+        if (!MPA_DBG_OK(dbg, sn + j, sizeof(ScanNode))) return;
+        const ScanNode& s = sn[j];
+        da = phase_q64(ka, s.da_hi, s.da_lo, s.db_hi, s.db_lo);
+        db = phase_q64(kb, s.da_hi, s.da_lo, s.db_hi, s.db_lo);
+        fresh = s.next;
     }
+    // (pre, pre, post, post) of node j
+    __device__ __forceinline__ float4 consts(int j) const {
+        const float4* a = reinterpret_cast<const float4*>(sn[j].pre);
+        return MPA_DBG_OK(dbg, a, 16) ? __ldg(a) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    // exp(i beta_j) at both frequencies, then on to node j + 1
+    __device__ __forceinline__ void next(float2& ea, float2& eb) {
+        expi_turns_poly2(ta, tb, ea, eb);
+        ta += da;
+        tb += db;
+    }
+};
+__device__ __forceinline__ float2 f4a(float4 v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 f4b(float4 v) { return make_float2(v.z, v.w); }
+__device__ __forceinline__ float4 f4(float2 a, float2 b) { return make_float4(a.x, a.y, b.x, b.y); }
+
+// The FP32 scan: a thread walks all nodes of two frequencies; its nodes
+// travel SCAN_S ahead through its own shared-memory slots by 16-byte
+// cp.async, so the bytes in flight do not cost registers.  STORE: mode 0.
+// 16 slots and five blocks an SM: 266 us a level at 2^20 x 126 nodes (the
+// scan without phases 261 us: the phases hide behind HBM), 126 us at 2^16 x
+// 801; 8 slots and eight blocks 270 and 140 us.
+constexpr int SCAN_S = 16, SCAN_NT = 128;
+template <bool STORE> __global__ void __launch_bounds__(SCAN_NT, 5) scan_pair_kernel(const ScanParams<float> p) {
+    __shared__ float4 ring[SCAN_S * SCAN_NT];
+    __shared__ float4 cst[SCAN_NT];  // PairWalk::consts of the nodes at hand
+    const int l = blockIdx.y;
+    const long long i = 2 * ((long long)blockIdx.x * SCAN_NT + threadIdx.x);
+    const long long lo = (long long)l * p.N, N2 = p.N >> 1;  // N2: float4 distance of nodes
+    float4* psi = reinterpret_cast<float4*>(p.psi + lo * (p.M + 1) + i);
+    // a pair shares a row of the tile layout, so its frequencies are neighbours there too
+    const long long k = p.tile_logG > 0 ? tile_to_natural(i, p.tile_logG, p.tile_logL, p.N) : i;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4* mine = ring + threadIdx.x;
+    const float4* ld = psi;
+#pragma unroll
+    for (int u = 0; u < SCAN_S; ++u) {
+        ld += N2;
+        if (1 + u <= p.M && MPA_DBG_OK(p.dbg, ld, 16)) cp_async16(mine + u * SCAN_NT, ld);
+        cp_async_commit();
+    }
+    const float4 v0 = MPA_DBG_OK(p.dbg, psi, 16) ? *psi : zero;
+    const float4* p0p = reinterpret_cast<const float4*>(p.psi0c + lo + k);
+    const float4 p0 = MPA_DBG_OK(p.dbg, p0p, 16) ? *p0p : zero;
+    const float2 pa = f4a(p0), pb = f4b(p0);
+    PairWalk walk(p, l, k);
+    // node 0: phase 0 and factor 1, V_0 = sigma_0 dz F_0
+    const float2 post0 = f4b(walk.consts(0));
+    float2 va = mul2(f4a(v0), post0), vb = mul2(f4b(v0), post0);
+    const float2 half = make_float2(0.5f, 0.5f);
+    float2 ra = mul2(va, half), rb = mul2(vb, half), ca = make_float2(0.f, 0.f), cb = ca;
+    walk.step(0);
+    walk.ta = walk.da;  // node 1
+    walk.tb = walk.db;
+    if (walk.fresh == 1) walk.step(1);
+    float2 na, nb;
+    walk.next(na, nb);
+    float4* st = psi;
+    int slot = 0;
+    for (int jb = 1; jb <= p.M; jb += SCAN_NT) {
+        // the factors of the next SCAN_NT nodes
+        const int je = p.M + 1 - jb < SCAN_NT ? p.M + 1 : jb + SCAN_NT;
+        __syncthreads();
+        if (jb + (int)threadIdx.x < je) cst[threadIdx.x] = walk.consts(jb + (int)threadIdx.x);
+        __syncthreads();
+        for (int j = jb; j < je;) {
+            // the loop takes the step from node j + 1 on: up to the node before the next change
+            if (j + 1 == walk.fresh) walk.step(j + 1);
+            // (any other value of fresh takes the rest of the nodes: the loop always advances)
+            const int end = walk.fresh > j + 1 && walk.fresh <= je ? walk.fresh - 1 : je;
+#pragma unroll 2
+            for (; j < end; ++j) {
+                const float4 w = cst[j - jb];
+                const float2 ea = na, eb = nb;
+                walk.next(na, nb);  // node j + 1's phases, beside node j's sums
+                cp_async_wait_group<SCAN_S - 1>();  // node j's copy has landed
+                float4* sl = mine + slot * SCAN_NT;
+                const float4 v = *sl;
+                slot = (slot + 1) & (SCAN_S - 1);
+                ld += N2;
+                st += N2;
+                va = mul2(cmul(f4a(v), cconj(ea)), f4b(w));
+                vb = mul2(cmul(f4b(v), cconj(eb)), f4b(w));
+                if constexpr (STORE) {
+                    // psi^{(n+1)}_j = psi_0 + i (R + V_j/2), stored with its phase and loss
+                    const float2 ha = fma2(va, half, csub(ra, ca)), hb = fma2(vb, half, csub(rb, cb));
+                    const float2 oa = cmul(make_float2(pa.x - ha.y, pa.y + ha.x), mul2(ea, f4a(w)));
+                    const float2 ob = cmul(make_float2(pb.x - hb.y, pb.y + hb.x), mul2(eb, f4a(w)));
+                    if (MPA_DBG_OK(p.dbg, st, 16)) *st = f4(oa, ob);
+                }
+                scan_add(ra, ca, va);
+                scan_add(rb, cb, vb);
+                // the slot's value is consumed: refill it with node j + SCAN_S
+                if (j + SCAN_S <= p.M && MPA_DBG_OK(p.dbg, ld, 16)) cp_async16(sl, ld);
+                cp_async_commit();
+            }
+        }
+    }
+    cp_async_wait_group<0>();
+    // D = R_M - V_M/2 at node M in FP64 (psi_M = psi_0 + i D)
+    scan_pair_m<true>(p, l, i, k, pa, pb, ((double)ra.x - (double)ca.x) - 0.5 * (double)va.x,
+                      ((double)ra.y - (double)ca.y) - 0.5 * (double)va.y, ((double)rb.x - (double)cb.x) - 0.5 * (double)vb.x,
+                      ((double)rb.y - (double)cb.y) - 0.5 * (double)vb.y, gridDim.x);
 }
 
 // The scan with the nodes of a frequency split over the block: 32 frequencies

@@ -12,7 +12,7 @@
 // step 4 mirrors it:
 //   V(p + P r) = sum_m W_C^{m r} W_N^{m p} sum_q W_P^{q p} U(C q + m).
 // The phases exp(+-i beta_j) and the Eq. (6) weight are applied at the load
-// and the store as in kn_kernel.  Every CTA of a cluster passes the same four
+// (PIN) and the store (POUT) as in kn_kernel.  Every CTA of a cluster passes the same four
 // cluster barriers (hardware barriers; no CTA leaves early).
 #pragma once
 
@@ -74,7 +74,7 @@ __device__ __forceinline__ void cluster_dft_rows(float2 (&out)[32], const unsign
     }
 }
 
-template <int C>
+template <int C, bool PIN, bool POUT>
 __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(512, 1) knc_kernel(const KNParams<float> p) {
     namespace cg = cooperative_groups;
     typedef KNCGeom<C> Gm;
@@ -110,14 +110,22 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(512, 1) knc_kernel(c
         const int l = node / p.npl, jn = node - l * p.npl;
         const float2* src =
             (p.src0 && jn == 0) ? p.src0 + l * p.src0_lstride : p.src + l * p.src_lstride + jn * p.src_stride;
-        const NodeC nc = p.nodes[p.loff[l] + jn];
-        PhaseRun pr(kf, 512, nc);
-        const float pre = (float)nc.pre;
+        if constexpr (PIN) {
+            const NodeC nc = p.nodes[p.loff[l] + jn];
+            PhaseRun pr(kf, 512, nc);
+            const float pre = (float)nc.pre;
 #pragma unroll
-        for (int r = 0; r < 32; ++r) {
-            const int pp = tid + 512 * r;
-            const float2 v = src[(long long)m * P + pp];
-            s[phys<Pt::PSH>(pp)] = cscale(cmul(v, expi_turns_poly(pr.next())), pre);
+            for (int r = 0; r < 32; ++r) {
+                const int pp = tid + 512 * r;
+                const float2 v = src[(long long)m * P + pp];
+                s[phys<Pt::PSH>(pp)] = cscale(cmul(v, expi_turns_poly(pr.next())), pre);
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < 32; ++r) {
+                const int pp = tid + 512 * r;
+                s[phys<Pt::PSH>(pp)] = src[(long long)m * P + pp];
+            }
         }
     }
     cl.sync();
@@ -156,22 +164,27 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(512, 1) knc_kernel(c
         s[phys<Pt::PSH>(pp)] = cmul(vout[0][r], cmul(whi[pp >> 7], wlo[pp & 127]));
     }
     cl.sync();
-    // ---- length-C forward DFT across the cluster (this CTA's slice m),
-    // V_j = F[U] exp(-i beta_j) sigma_j dz / exp(int G)  (Eq. (6))
+    // ---- length-C forward DFT across the cluster (this CTA's slice m)
     {
         const int l = node / p.npl, jn = node - l * p.npl;
         float2* dst = p.dst + l * p.dst_lstride + jn * p.dst_stride;
-        const NodeC nc = p.nodes[p.loff[l] + jn];
         unsigned rs[C];
 #pragma unroll
         for (int c = 0; c < C; ++c) rs[c] = cluster_smem_addr(s + phys<Pt::PSH>(tid), (unsigned)c);
         cluster_dft_rows<C, +1, 0>(vout[0], rs, m);
-        PhaseRun pr(kf, 512, nc);
-        const float post = (float)nc.post;
+        if constexpr (POUT) {
+            // V_j = F[U] exp(-i beta_j) sigma_j dz / exp(int G)  (Eq. (6))
+            const NodeC nc = p.nodes[p.loff[l] + jn];
+            PhaseRun pr(kf, 512, nc);
+            const float post = (float)nc.post;
 #pragma unroll
-        for (int r = 0; r < 32; ++r) {
-            const int pp = tid + 512 * r;
-            dst[(long long)m * P + pp] = cscale(cmul(vout[0][r], cconj(expi_turns_poly(pr.next()))), post);
+            for (int r = 0; r < 32; ++r) {
+                const int pp = tid + 512 * r;
+                dst[(long long)m * P + pp] = cscale(cmul(vout[0][r], cconj(expi_turns_poly(pr.next()))), post);
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < 32; ++r) dst[(long long)m * P + tid + 512 * r] = vout[0][r];
         }
     }
     cl.sync();  // keep this slice alive until every partner has read it

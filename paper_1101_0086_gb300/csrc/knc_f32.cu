@@ -4,19 +4,19 @@
 
 namespace mpa {
 
-template <int C>
+template <int C, bool PIN, bool POUT>
 static cudaError_t knc_one(const KNParams<float>& p, cudaStream_t st) {
     if (const cudaError_t eg = launch_gate()) return eg;
     typedef KNCGeom<C> Gm;
     static AttrOnce once;
     const cudaError_t ea = attrs_once(once, [] {
-        return cudaFuncSetAttribute(knc_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Gm::smem_bytes);
+        return cudaFuncSetAttribute(knc_kernel<C, PIN, POUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Gm::smem_bytes);
     });
     if (ea != cudaSuccess) return ea;
     if (p.nrows <= 0) return cudaSuccess;
     const bool prof = g_prof_on.load(std::memory_order_relaxed);
     if (prof) prof_begin(st);
-    knc_kernel<C><<<(unsigned)(p.nrows * C), Gm::NT, Gm::smem_bytes, st>>>(p);
+    knc_kernel<C, PIN, POUT><<<(unsigned)(p.nrows * C), Gm::NT, Gm::smem_bytes, st>>>(p);
     if (prof) {
         const double cs = (double)sizeof(float2), nodes = (double)p.nrows, L = (double)C * Gm::P;
         const double rd = p.src_stride == 0 ? nodes / p.npl : nodes;
@@ -26,10 +26,15 @@ static cudaError_t knc_one(const KNParams<float>& p, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+template <int C> static cudaError_t knc_len(const KNParams<float>& p, cudaStream_t st) {
+    if (p.phase_out) return p.phase_in ? knc_one<C, true, true>(p, st) : cudaErrorInvalidValue;
+    return p.phase_in ? knc_one<C, true, false>(p, st) : knc_one<C, false, false>(p, st);
+}
+
 cudaError_t knc_launch(int logL, const KNParams<float>& p, cudaStream_t st) {
     switch (logL) {
-        case 15: return knc_one<2>(p, st);
-        case 16: return knc_one<4>(p, st);
+        case 15: return knc_len<2>(p, st);
+        case 16: return knc_len<4>(p, st);
     }
     return cudaErrorInvalidValue;
 }

@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(KNGeom<float, L>::NT, 1) kp_kernel(const KPPar
             k.nodes = p.nodes;
             k.loff = loff;
             k.inv_n = p.inv_n;
-            kn_tile<float, L, true>(k, (long long)idx * G, smem_raw);
+            kn_tile<float, L, true, true, true>(k, (long long)idx * G, smem_raw);
         } else {
             ScanParams<float> s{};
             s.psi = p.psi + l * npl * N;
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(KNGeom<float, L>::NT, 1) kp_kernel(const KPPar
             s.level = (int)n;
             s.n_iter = p.n_iter;
             s.floor_rel = p.floor_rel;
-            scan_freq<float, true>(s, 0, (long long)idx * NT + tid, (unsigned)p.ns);
+            scan_freq<float, true, false>(s, 0, (long long)idx * NT + tid, (unsigned)p.ns);
         }
         // this task's writes are visible before it is counted
         __threadfence();

@@ -53,7 +53,8 @@ enum {
 extern std::atomic<bool> g_prof_on;
 void prof_begin(cudaStream_t st);
 void prof_end(int kind, cudaStream_t st, double bytes);
-int prof_kc_kind(int mode);
+// levels: a pass of the MPA levels (its transforms count with the MPA passes)
+int prof_kc_kind(int mode, bool levels);
 // Per-call timer of the entry points (mpa_last_timing): while profiling is
 // on, the outermost timed entry point of a thread records a CUDA event on
 // its stream at construction and at destruction (not on a capturing stream).

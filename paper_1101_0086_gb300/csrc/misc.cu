@@ -152,7 +152,8 @@ cudaError_t call_timing_read(double* ms, const char** entry, bool* have) {
     return cudaSuccess;
 }
 
-int prof_kc_kind(int mode) {
+int prof_kc_kind(int mode, bool levels) {
+    if (levels && (mode == KC_INV || mode == KC_FWD)) return mode == KC_INV ? PK_KC_MPA_PRE : PK_KC_MPA_POST;
     return mode == KC_MPA_PRE ? PK_KC_MPA_PRE : mode == KC_MPA_POST ? PK_KC_MPA_POST
          : mode == KC_SS_STEP ? PK_KC_SS : PK_KC_FFT;
 }
@@ -181,21 +182,27 @@ void prof_reset() {
 
 static unsigned blocks_for(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
-// Frequencies (N x links) up to which a scan splits its nodes over the block
-// (scan_split_kernel).  Measured, us a launch, split / unsplit: FP32, 143
-// nodes: 2^12 13.5 / 20.9, 2^14 17.7 / 20.6, 2^15 24.5 / 21.7; 801 nodes:
-// 2^12 21 / 63, 2^14 43 / 80.  FP64 is bound by its adds, which the split
-// form doubles: 143 nodes 2^12 24 / 54, 2^13 37 / 54.
-template <typename T> constexpr long long scan_split_max() { return sizeof(T) == 4 ? 1ll << 14 : 1ll << 13; }
+// Frequencies (N x links) up to which an FP64 scan splits its nodes over the
+// block (scan_split_kernel).  FP64 is bound by its adds, which the split form
+// doubles: 143 nodes, us a launch, split / unsplit: 2^12 24 / 54, 2^13 37 /
+// 54.  FP32 scans split wherever the node transforms apply the phases
+// (scan_phases_min).
+constexpr long long kScanSplit64Max = 1ll << 13;
 
 template <typename T> cudaError_t scan_launch(const ScanParams<T>& p, int p_links, cudaStream_t st) {
     if (const cudaError_t eg = launch_gate()) return eg;
     const bool pr = g_prof_on.load(std::memory_order_relaxed);
     if (pr) prof_begin(st);
-    if (p.N * p_links <= scan_split_max<T>())
-        scan_split_kernel<T><<<dim3(blocks_for(p.N, 32), (unsigned)p_links), 32 * SCS_W, 0, st>>>(p);
-    else
-        scan_kernel<T><<<dim3(blocks_for(p.N, 256), (unsigned)p_links), 256, 0, st>>>(p);
+    const dim3 grid(blocks_for(p.N, 256), (unsigned)p_links), split(blocks_for(p.N, 32), (unsigned)p_links);
+    if constexpr (sizeof(T) == 4) {
+        if (!p.phases) scan_split_kernel<T><<<split, 32 * SCS_W, 0, st>>>(p);
+        else if (p.mode == 0) scan_pair_kernel<true><<<grid, SCAN_NT, 0, st>>>(p);
+        else scan_pair_kernel<false><<<grid, SCAN_NT, 0, st>>>(p);
+    } else {
+        if (p.phases) scan_kernel<T, true><<<grid, 256, 0, st>>>(p);
+        else if (p.N * p_links <= kScanSplit64Max) scan_split_kernel<T><<<split, 32 * SCS_W, 0, st>>>(p);
+        else scan_kernel<T, false><<<grid, 256, 0, st>>>(p);
+    }
     if (pr) {
         const double cs = (double)sizeof(cx<T>), n = (double)p.N;
         double b = ((p.M + 1) * n * cs + n * cs) * p_links;  // V_0..V_M and psi_0

@@ -1,6 +1,7 @@
 // C ABI of the MPA / split-step library: plan creation (host tables of the
 // per-node constants of Eq. (6)), workspace layout, and the launch schedule
 // of the MPA steps 1-7 and of the split-step of Eq. (4).
+#include <climits>
 #include <cmath>
 #include <cstddef>
 #include <cstdio>
@@ -36,12 +37,27 @@ namespace host {
 // interval; gain[l] is its amplifier gain at the interval end (device).
 // Every iteration covers nodes 0..M of every link; node 0 always reads
 // psi_0, so V_0 (identical at every iteration) is simply recomputed.
+// Frequencies (N x links) from which the scan applies the phases of steps 2
+// and 5 (ScanParams::phases) instead of the node transforms' load and store.
+// A level in us, with / without: FP32, 143 nodes: 2^14 42.0 / 42.8, 2^15 83 /
+// 93, 2^16 (four-step) 138 / 156, 2^18 453 / 512, 2^20 1671 / 1846; 801
+// nodes: 2^14 172 / 181, 2^16 702 / 762.  FP64 (every phase a full
+// evaluation in the scan too): 2^14 1349 / 1185, 2^15 2087 / 2173, 2^16
+// 4134 / 4357.
+template <typename T> constexpr long long scan_phases_min() { return sizeof(T) == 4 ? 1ll << 14 : 1ll << 15; }
+
+// With ph (many frequencies), psi holds A_hat_j before the node transforms
+// (level 0 reads psi_0 and applies the phases at the load) and F_j =
+// F[|A_j|^2 A_j] after them, and the scan turns F_j into the next level's
+// A_hat_j: one phase evaluation per node and frequency, in the kernel that
+// waits for memory, instead of two in passes that wait for issue slots.
 template <typename T>
 int mpa_levels(const Split& s, int M, int n_iter, int nl, cx<T>* psi, cx<T>* work, cx<T>* psi0c, double2* state,
-               const NodeC* nodes, const int* loff, const double* gain, const Monitor& mon, int scan_mode,
-               double2* out, cudaStream_t st) {
+               const NodeC* nodes, const ScanNode* scn, const int* loff, const double* gain, const Monitor& mon,
+               int scan_mode, double2* out, cudaStream_t st) {
     const long long N = s.N;
     const int npl = M + 1;
+    const bool ph = N * nl >= scan_phases_min<T>();
     int tile_log_g = 0;  // > 0: node spectra between the passes in the staged column pass's tile layout
     for (int n = 0; n < n_iter; ++n) {
         if (s.onchip) {
@@ -60,6 +76,8 @@ int mpa_levels(const Split& s, int M, int n_iter, int nl, cx<T>* psi, cx<T>* wor
             k.nodes = nodes;
             k.loff = loff;
             k.inv_n = (T)(1.0 / (double)N);
+            k.phase_in = !ph || n == 0;
+            k.phase_out = !ph;
             k.dbg = mon.dbg;
             MPA_TRY(kn_launch<T>(s.logN, k, st));
         } else {
@@ -85,15 +103,15 @@ int mpa_levels(const Split& s, int M, int n_iter, int nl, cx<T>* psi, cx<T>* wor
         c.spin_limit = mon.spin_limit;
         c.dbg = mon.dbg;
         if constexpr (sizeof(T) == 4)
-            tile_log_g = work && kc_staged(KC_MPA_POST, s.logN2, c) ? kcs_tile_log_cols(s.logN2) : 0;
-        // Tile layout: the forward pass writes V_j into psi in the tile layout
-        // of the staged column pass, the scan keeps it for psi^{(n+1)}, and the
+            tile_log_g = ph && work && kc_staged(KC_FWD, s.logN2, c) ? kcs_tile_log_cols(s.logN2) : 0;
+        // Tile layout: the forward pass writes F_j into psi in the tile layout
+        // of the staged column pass, the scan keeps it for A_hat_j, and the
         // next inverse pass reads whole tiles from psi and writes the natural
         // order into `work`, where the row pass and the forward pass run.
         cx<T>* xw = tile_log_g > 0 ? work : psi;
         c.tiled_in = n > 0 && tile_log_g > 0;
         c.dst = xw;
-        MPA_TRY(kc_launch<T>(KC_MPA_PRE, s.logN2, c, st));
+        MPA_TRY(kc_launch<T>(!ph || n == 0 ? KC_MPA_PRE : KC_INV, s.logN2, c, st));
         KRParams<T> r{xw, (long long)nl * npl * s.N2, N, s.logN, (int)s.N2, (T)(1.0 / (double)N), T(0)};
         r.err = mon.err;
         r.spin_limit = mon.spin_limit;
@@ -106,7 +124,7 @@ int mpa_levels(const Split& s, int M, int n_iter, int nl, cx<T>* psi, cx<T>* wor
         c.dst = psi;
         c.tiled_in = 0;
         c.tiled_out = tile_log_g > 0;
-        MPA_TRY(kc_launch<T>(KC_MPA_POST, s.logN2, c, st));
+        MPA_TRY(kc_launch<T>(ph ? KC_FWD : KC_MPA_POST, s.logN2, c, st));
         }
         // step 5 (Eq. (6)); on the last iteration fused with step 7
         ScanParams<T> q{};
@@ -119,6 +137,8 @@ int mpa_levels(const Split& s, int M, int n_iter, int nl, cx<T>* psi, cx<T>* wor
         q.out = out;
         q.mode = (n == n_iter - 1) ? scan_mode : 0;
         q.nodes = nodes;
+        q.scn = scn;
+        q.phases = ph;
         q.loff = loff;
         q.gain = gain;
         q.err = mon.err;
@@ -136,9 +156,46 @@ int mpa_levels(const Split& s, int M, int n_iter, int nl, cx<T>* psi, cx<T>* wor
 }
 
 template int mpa_levels<float>(const Split&, int, int, int, float2*, float2*, float2*, double2*, const NodeC*,
-                               const int*, const double*, const Monitor&, int, double2*, cudaStream_t);
+                               const ScanNode*, const int*, const double*, const Monitor&, int, double2*, cudaStream_t);
 template int mpa_levels<double>(const Split&, int, int, int, double2*, double2*, double2*, double2*, const NodeC*,
-                                const int*, const double*, const Monitor&, int, double2*, cudaStream_t);
+                                const ScanNode*, const int*, const double*, const Monitor&, int, double2*,
+                                cudaStream_t);
+
+void scan_nodes(const HostMap& m, double u0, double L, int M, double T, const NodeC* nodes, std::vector<ScanNode>* out) {
+    const double dz = L / M;
+    const size_t base = out->size();
+    double p2 = 0.0, p3 = 0.0;
+    int open = 0;  // the first node of the current run of equal steps
+    for (int j = 0; j <= M; ++j) {
+        ScanNode c{};
+        c.pre[0] = c.pre[1] = (float)nodes[j].pre;
+        c.post[0] = c.post[1] = (float)nodes[j].post;
+        c.next = INT_MAX;  // none
+        if (j < M) {
+            const double za = u0 + dz * j, zb = u0 + (j + 1 == M ? L : dz * (j + 1));
+            // within one segment the step is its coefficient times dz, free of the
+            // rounding of the node positions and the same at every node
+            auto step = [&](int col) {
+                const double x = m.integ(za, zb, col), y = m.side(za, col, +1) * dz;
+                return std::fabs(x - y) <= 1e-9 * std::fabs(y) ? y : x;
+            };
+            const double s2 = step(1), s3 = step(2);
+            NodeC t{};
+            phase_consts(s2, s3, T, &t);
+            c.da_hi = t.a_hi;
+            c.da_lo = t.a_lo;
+            c.db_hi = t.b_hi;
+            c.db_lo = t.b_lo;
+            if (j > 0 && (s2 != p2 || s3 != p3)) {
+                for (int q = open; q < j; ++q) (*out)[base + (size_t)q].next = j;
+                open = j;
+            }
+            p2 = s2;
+            p3 = s3;
+        }
+        out->push_back(c);
+    }
+}
 
 }  // namespace host
 }  // namespace mpa
@@ -180,7 +237,8 @@ int run_interval(mpa_plan* p, int type, long n_amp, int scan_mode, double2* out,
                          p->has_work ? reinterpret_cast<cx<T>*>(p->ws + p->off_work2) : nullptr,
                          reinterpret_cast<cx<T>*>(p->ws + p->off_psi0c),
                          reinterpret_cast<double2*>(p->ws + p->off_state),
-                         reinterpret_cast<const NodeC*>(p->ws + p->off_nodes), toff + type, gains + n_amp,
+                         reinterpret_cast<const NodeC*>(p->ws + p->off_nodes),
+                         reinterpret_cast<const ScanNode*>(p->ws + p->off_scn), toff + type, gains + n_amp,
                          monitor(p), scan_mode, out, st);
 }
 template int run_interval<float>(mpa_plan*, int, long, int, double2*, cudaStream_t);
@@ -475,7 +533,13 @@ int mpa_plan_create(const mpa_fiber_map* map, const mpa_plan_params* prm, mpa_pl
         const size_t after_psi0c =
             p->prec == MPA_FP32 ? p->off_psi0c + psi0c_bytes : p->off_state + N * sizeof(double2);
         p->off_nodes = align256(after_psi0c);
-        p->off_toff = align256(p->off_nodes + p->nodes.size() * sizeof(NodeC));
+        if (p->prec == MPA_FP32) {
+            p->scn.reserve(p->nodes.size());
+            for (int t = 0; t < p->n_types; ++t)
+                scan_nodes(p->map, p->L * t, p->L, M, p->T, p->nodes.data() + (size_t)t * (M + 1), &p->scn);
+        }
+        p->off_scn = align256(p->off_nodes + p->nodes.size() * sizeof(NodeC));
+        p->off_toff = align256(p->off_scn + p->scn.size() * sizeof(ScanNode));
         p->off_gains = align256(p->off_toff + (size_t)p->n_types * sizeof(int));
         p->off_err = align256(p->off_gains + kMaxAmpsPerInterval * sizeof(double));
         p->off_conv = align256(p->off_err + sizeof(unsigned int));
@@ -500,6 +564,9 @@ int mpa_plan_set_workspace(mpa_plan* p, void* ws, size_t bytes) {
         p->ws_bytes = bytes;
         MPA_TRY(cudaMemcpy(p->ws + p->off_nodes, p->nodes.data(), p->nodes.size() * sizeof(NodeC),
                            cudaMemcpyHostToDevice));
+        if (!p->scn.empty())
+            MPA_TRY(cudaMemcpy(p->ws + p->off_scn, p->scn.data(), p->scn.size() * sizeof(ScanNode),
+                               cudaMemcpyHostToDevice));
         std::vector<int> toff((size_t)p->n_types);
         for (int t = 0; t < p->n_types; ++t) toff[(size_t)t] = t * (p->M + 1);
         MPA_TRY(cudaMemcpy(p->ws + p->off_toff, toff.data(), toff.size() * sizeof(int), cudaMemcpyHostToDevice));

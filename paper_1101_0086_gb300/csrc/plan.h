@@ -14,6 +14,8 @@ struct mpa_plan {
     int M, n_iter, prec;
     int n_types;                // distinct interval starts within the DM period
     std::vector<mpa::NodeC> nodes;  // n_types x (M+1)
+    std::vector<mpa::ScanNode> scn; // n_types x (M+1), FP32 level-schedule plans
+    size_t off_scn = 0;
     size_t csize;               // bytes per complex sample
     size_t off_psi, off_state, off_psi0c, off_nodes, off_err, off_toff, off_gains, ws_need;
     size_t off_conv = 0, off_dprev = 0;  // Picard increment check (ConvState, D at node M)
