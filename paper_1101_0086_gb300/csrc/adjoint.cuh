@@ -26,6 +26,7 @@
 // CTAs per SM the reverse passes are compiled for (1: up to 255 registers,
 // no spills; 2: 128 registers, a few spills): 2 for both, measured faster
 // (MPA reverse column passes 3.10 -> 3.99 TB/s, row pass 2.36 -> 2.81 TB/s).
+// FP64 passes, bound by FP64 instructions, take 1.
 #ifndef MPA_ADJ_MINB
 #define MPA_ADJ_MINB 2
 #endif
@@ -120,7 +121,7 @@ template <typename T> __device__ __forceinline__ T ksq(long long kk) {
 }
 
 template <typename T, int L, int MODE>
-__global__ void __launch_bounds__(KCGeom<T, L>::NT, KCGeom<T, L>::NT <= 256 ? MPA_ADJ_MINB : 1) kca_kernel(const KCAParams<T> p) {
+__global__ void __launch_bounds__(KCGeom<T, L>::NT, KCGeom<T, L>::NT <= 256 && sizeof(T) == 4 ? MPA_ADJ_MINB : 1) kca_kernel(const KCAParams<T> p) {
     typedef cx<T> C;
     typedef KCGeom<T, L> Gm;
     typedef Tiling<T> P;
@@ -134,7 +135,7 @@ __global__ void __launch_bounds__(KCGeom<T, L>::NT, KCGeom<T, L>::NT <= 256 ? MP
     C* s = reinterpret_cast<C*>(smem_raw);
     C* thi = s + TE + (TE >> P::PSH) + 1;
     C* tlo = thi + TwDims<L>::NHI;
-    C* olo = tlo + TwDims<L>::NLO;
+    C* olo = thi + Tw<T, L>::N;
     C* ohi = olo + G * Gm::OLO;
     const int tid = threadIdx.x;
     const long long col0 = (long long)blockIdx.x * G;
@@ -178,7 +179,7 @@ __global__ void __launch_bounds__(KCGeom<T, L>::NT, KCGeom<T, L>::NT <= 256 ? MP
                 acc.add(ksq<T>(kk) * im_conj_mul(v, aux[idx]));
                 C ph;
                 if constexpr (FAST) ph = expi_turns_poly(pr.next());
-                else ph = expi_turns<T>(phase_q64(kk, nc));
+                else ph = expi_at<T, L>(phase_q64(kk, nc), thi);
                 v = cscale(cmul(v, ph), (T)ac.dzp);
             }
             vin[q][r] = v;
@@ -213,7 +214,7 @@ __global__ void __launch_bounds__(KCGeom<T, L>::NT, KCGeom<T, L>::NT <= 256 ? MP
                 const long long kk = signed_k(idx, p.N);
                 C ph;
                 if constexpr (FAST) ph = expi_turns_poly(pr.next());
-                else ph = expi_turns<T>(phase_q64(kk, nc));
+                else ph = expi_at<T, L>(phase_q64(kk, nc), thi);
                 v = cscale(cmul(v, cconj(ph)), post);
                 acc.add(-ksq<T>(kk) * im_conj_mul(v, aux[idx]));
             }
@@ -225,7 +226,7 @@ __global__ void __launch_bounds__(KCGeom<T, L>::NT, KCGeom<T, L>::NT <= 256 ? MP
 }
 
 template <typename T, int L>
-__global__ void __launch_bounds__(KRGeom<T, L>::NT, KRGeom<T, L>::NT <= 256 ? MPA_ADJ_MINB_R : 1) kra_kernel(const KRAParams<T> p) {
+__global__ void __launch_bounds__(KRGeom<T, L>::NT, KRGeom<T, L>::NT <= 256 && sizeof(T) == 4 ? MPA_ADJ_MINB_R : 1) kra_kernel(const KRAParams<T> p) {
     typedef cx<T> C;
     typedef KRGeom<T, L> Gm;
     typedef Tiling<T, 1> P;
@@ -238,7 +239,7 @@ __global__ void __launch_bounds__(KRGeom<T, L>::NT, KRGeom<T, L>::NT <= 256 ? MP
     C* s = reinterpret_cast<C*>(smem_raw);
     C* thi = s + TE + (TE >> P::PSH) + 1;
     C* tlo = thi + TwDims<L>::NHI;
-    C* olo = tlo + TwDims<L>::NLO;
+    C* olo = thi + Tw<T, L>::N;
     C* ohi = olo + G * Gm::OLO;
     const int tid = threadIdx.x;
     const long long row0 = (long long)blockIdx.x * G;
@@ -474,7 +475,7 @@ template <typename T> struct SSRParams {
 };
 
 template <typename T, int L, int MODE>
-__global__ void __launch_bounds__(KCGeom<T, L>::NT, KCGeom<T, L>::NT <= 256 ? MPA_ADJ_MINB : 1) ssc_kernel(const SSCParams<T> p) {
+__global__ void __launch_bounds__(KCGeom<T, L>::NT, KCGeom<T, L>::NT <= 256 && sizeof(T) == 4 ? MPA_ADJ_MINB : 1) ssc_kernel(const SSCParams<T> p) {
     typedef cx<T> C;
     typedef KCGeom<T, L> Gm;
     typedef Tiling<T> P;
@@ -487,7 +488,7 @@ __global__ void __launch_bounds__(KCGeom<T, L>::NT, KCGeom<T, L>::NT <= 256 ? MP
     C* s = reinterpret_cast<C*>(smem_raw);
     C* thi = s + TE + (TE >> P::PSH) + 1;
     C* tlo = thi + TwDims<L>::NHI;
-    C* olo = tlo + TwDims<L>::NLO;
+    C* olo = thi + Tw<T, L>::N;
     C* ohi = olo + G * Gm::OLO;
     const int tid = threadIdx.x;
     const long long col0 = (long long)blockIdx.x * G;
@@ -527,7 +528,7 @@ __global__ void __launch_bounds__(KCGeom<T, L>::NT, KCGeom<T, L>::NT <= 256 ? MP
             const long long idx = c + (long long)(j + r * (L / XF::RL)) * p.N1;
             C ph;
             if constexpr (FAST) ph = expi_turns_poly(th[r]);
-            else ph = expi_turns<T>(phase_q64(signed_k(idx, p.N), p.flow));
+            else ph = expi_at<T, L>(phase_q64(signed_k(idx, p.N), p.flow), thi);
             if constexpr (MODE == SS_REV) acc.add(-ksq<T>(signed_k(idx, p.N)) * im_conj_mul(vm[q][r], p.xs[idx]));
             vm[q][r] = cscale(cmul(vm[q][r], ph), (T)p.pre);
             if constexpr (MODE == SS_STORE) p.xs[idx] = vm[q][r];
@@ -557,7 +558,7 @@ __global__ void __launch_bounds__(KCGeom<T, L>::NT, KCGeom<T, L>::NT <= 256 ? MP
 }
 
 template <typename T, int L, int MODE>
-__global__ void __launch_bounds__(KRGeom<T, L>::NT, KRGeom<T, L>::NT <= 256 ? MPA_ADJ_MINB_R : 1) ssr_kernel(const SSRParams<T> p) {
+__global__ void __launch_bounds__(KRGeom<T, L>::NT, KRGeom<T, L>::NT <= 256 && sizeof(T) == 4 ? MPA_ADJ_MINB_R : 1) ssr_kernel(const SSRParams<T> p) {
     typedef cx<T> C;
     typedef KRGeom<T, L> Gm;
     typedef Tiling<T, 1> P;
@@ -570,7 +571,7 @@ __global__ void __launch_bounds__(KRGeom<T, L>::NT, KRGeom<T, L>::NT <= 256 ? MP
     C* s = reinterpret_cast<C*>(smem_raw);
     C* thi = s + TE + (TE >> P::PSH) + 1;
     C* tlo = thi + TwDims<L>::NHI;
-    C* olo = tlo + TwDims<L>::NLO;
+    C* olo = thi + Tw<T, L>::N;
     C* ohi = olo + G * Gm::OLO;
     const int tid = threadIdx.x;
     const long long row0 = (long long)blockIdx.x * G;

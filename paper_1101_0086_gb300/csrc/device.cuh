@@ -133,37 +133,40 @@ template <int R, int K, int S, class C> __device__ __forceinline__ C tw_const(C 
     }
 }
 
-// FP32 butterflies with a non-trivial constant twiddle (K/R not a multiple
-// of 1/4) as fused multiply-adds: x0 = e + w o with the twiddle's products
-// folded into the additions, x1 = 2 e - x0 (= e - w o): six FP32 operations
-// instead of eight (two products, two fused products and four additions).
-// The difference from x1 = e - w o is one rounding of x0, of the size of the
-// rounding of the product itself.  MPA_FMA_BFLY=0 keeps the plain form.
+// Butterflies with a non-trivial constant twiddle (K/R not a multiple of 1/4)
+// as fused multiply-adds: x0 = e + w o with the twiddle's products folded into
+// the additions, x1 = 2 e - x0 (= e - w o): six operations instead of eight
+// (two products, two fused products and four additions).  The difference from
+// x1 = e - w o is one rounding of x0, of the size of the rounding of the
+// product itself.  MPA_FMA_BFLY=0 keeps the plain form.
 #ifndef MPA_FMA_BFLY
 #define MPA_FMA_BFLY 1
 #endif
-template <int R, int K, int S> __device__ __forceinline__ void bfly_tw(float2& x0, float2& x1, float2 e, float2 o) {
+__device__ __forceinline__ float ffma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double ffma(double a, double b, double c) { return fma(a, b, c); }
+template <int R, int K, int S, class C> __device__ __forceinline__ void bfly_tw(C& x0, C& x1, C e, C o) {
+    typedef decltype(e.x) T;
     constexpr int M32 = K * (32 / R);
-    float ax, ay;
+    T ax, ay;
     if constexpr (M32 == 4 || M32 == 12) {
         // w = c (re + S i), c = cos(pi/4): x0 = e + c (re o.x - S o.y, re o.y + S o.x)
-        constexpr float re = (M32 == 4) ? 1.f : -1.f;
-        const float c = (float)MPA_COS_PI_4;
-        ax = fmaf(c, re * o.x - float(S) * o.y, e.x);
-        ay = fmaf(c, re * o.y + float(S) * o.x, e.y);
+        constexpr T re = (M32 == 4) ? T(1) : T(-1);
+        const T c = (T)MPA_COS_PI_4;
+        ax = ffma(c, re * o.x - T(S) * o.y, e.x);
+        ay = ffma(c, re * o.y + T(S) * o.x, e.y);
     } else {
-        const float cr = (float)Cs32<M32>::c, si = float(S) * (float)Cs32<M32>::s;
-        ax = fmaf(o.x, cr, fmaf(-o.y, si, e.x));
-        ay = fmaf(o.x, si, fmaf(o.y, cr, e.y));
+        const T cr = (T)Cs32<M32>::c, si = T(S) * (T)Cs32<M32>::s;
+        ax = ffma(o.x, cr, ffma(-o.y, si, e.x));
+        ay = ffma(o.x, si, ffma(o.y, cr, e.y));
     }
-    x0 = make_float2(ax, ay);
-    x1 = make_float2(fmaf(2.f, e.x, -ax), fmaf(2.f, e.y, -ay));
+    x0 = mkc(ax, ay);
+    x1 = mkc(ffma(T(2), e.x, -ax), ffma(T(2), e.y, -ay));
 }
 
 template <int R, int S, int K, class C> __device__ __forceinline__ void dft_combine(C* x, const C* e, const C* o) {
     if constexpr (K < R / 2) {
         constexpr int M32 = K * (32 / R);
-        if constexpr (MPA_FMA_BFLY && sizeof(C) == 8 && M32 != 0 && M32 != 8) {
+        if constexpr (MPA_FMA_BFLY && M32 != 0 && M32 != 8) {
             bfly_tw<R, K, S>(x[K], x[K + R / 2], e[K], o[K]);
         } else {
             const C t = tw_const<R, K, S>(o[K]);
@@ -526,6 +529,14 @@ template <int L> struct TwDims {
     static constexpr int NHI = L >> SH;
 };
 
+// FP64 transforms of up to 2048 points keep the whole table of W_L instead
+// (hi[e], no product per lookup): FP64 instructions are the bound of the
+// FP64 passes (1.7 a clock and SM), shared-memory reads are not.
+template <typename T, int L> struct Tw {
+    static constexpr bool FULL = sizeof(T) == 8 && L >= 16 && L <= 2048;
+    static constexpr int N = FULL ? L : TwDims<L>::NLO + TwDims<L>::NHI;  // entries in shared memory
+};
+
 // Slot of entry e of the low twiddle table.  A row-pass warp looks up
 // e = s j for 32 consecutive j and a power of two s; 8-byte entries sit in 16
 // bank pairs, so in natural order the stride s = 4, 8, 16 lookups would
@@ -538,16 +549,58 @@ template <int NLO> __device__ __forceinline__ int tw_lo_slot(int e) {
 
 template <typename T, int L> __device__ __forceinline__ void tw_init(cx<T>* hi, cx<T>* lo, int tid, int nt) {
     typedef TwDims<L> D;
-    for (int i = tid; i < D::NLO + D::NHI; i += nt) {
-        if (i < D::NLO) lo[tw_lo_slot<D::NLO>(i)] = expi_ratio<T>(i, D::logL);
-        else hi[i - D::NLO] = expi_ratio<T>((long long)(i - D::NLO) << D::SH, D::logL);
+    if constexpr (Tw<T, L>::FULL) {
+        // the first octant evaluated, the others its reflections (exact)
+        for (int m = tid; m <= L / 8; m += nt) {
+            const cx<T> w = expi_ratio<T>(m, D::logL);
+            hi[m] = w;
+            hi[L / 4 - m] = mkc(w.y, w.x);
+            hi[L / 4 + m] = mkc(-w.y, w.x);
+            hi[L / 2 - m] = mkc(-w.x, w.y);
+            hi[L / 2 + m] = mkc(-w.x, -w.y);
+            hi[3 * L / 4 - m] = mkc(-w.y, -w.x);
+            hi[3 * L / 4 + m] = mkc(w.y, -w.x);
+            if (m > 0) hi[L - m] = mkc(w.x, -w.y);
+        }
+    } else {
+        for (int i = tid; i < D::NLO + D::NHI; i += nt) {
+            if (i < D::NLO) lo[tw_lo_slot<D::NLO>(i)] = expi_ratio<T>(i, D::logL);
+            else hi[i - D::NLO] = expi_ratio<T>((long long)(i - D::NLO) << D::SH, D::logL);
+        }
     }
 }
 
 template <typename T, int L> __device__ __forceinline__ cx<T> tw_get(const cx<T>* hi, const cx<T>* lo, int e) {
     typedef TwDims<L> D;
-    if constexpr (D::NHI == 1) return lo[tw_lo_slot<D::NLO>(e)];
+    if constexpr (Tw<T, L>::FULL) return hi[e];
+    else if constexpr (D::NHI == 1) return lo[tw_lo_slot<D::NLO>(e)];
     else return cmul(hi[e >> D::SH], lo[tw_lo_slot<D::NLO>(e & (D::NLO - 1))]);
+}
+
+// exp(2 pi i theta) of a Q0.64 turn fraction in FP64 beside a full table of
+// W_L (256 <= L <= 2048): theta = m / L + x / (2 pi) with |x| <= pi / L, and
+// W_L^m (1 + (cos x - 1) + i sin x) by short Taylor series (the first dropped
+// terms, x^8/40320 and x^7/5040, are below 1.3e-20 and 8.4e-18): 13 FP64
+// instructions instead of a full-range sincospi, with the table's correctly
+// rounded entry entering last.  x comes from the integer's upper 51 bits by
+// the addition of 1.5 2^52 (exact), not by a conversion.
+template <int L> __device__ __forceinline__ double2 expi_tab(unsigned long long th, const double2* tab) {
+    constexpr int LG = TwDims<L>::logL, SH = 13 - LG;
+    static_assert(Tw<double, L>::FULL && L >= 256, "a full table of at least 256 entries");
+    const unsigned m = (unsigned)((th + (1ull << (63 - LG))) >> (64 - LG));  // nearest (wraps to 0)
+    const long long d = (long long)(th - ((unsigned long long)m << (64 - LG))) >> SH;  // |d| <= 2^50
+    const double x = (__longlong_as_double(0x4338000000000000ll + d) - 6755399441055744.0) *
+                     (3.4061215800865545e-19 * (double)(1 << SH));  // 2 pi 2^-64 2^SH
+    const double2 t = tab[m & (L - 1)];
+    const double x2 = x * x;
+    const double c = x2 * fma(x2, fma(x2, -1.0 / 720.0, 1.0 / 24.0), -0.5);
+    const double s = fma(x * x2, fma(x2, 1.0 / 120.0, -1.0 / 6.0), x);
+    return make_double2(fma(t.x, c, fma(-t.y, s, t.x)), fma(t.y, c, fma(t.x, s, t.y)));
+}
+// exp(2 pi i theta) in a kernel that holds the twiddle tables of W_L
+template <typename T, int L> __device__ __forceinline__ cx<T> expi_at(unsigned long long th, const cx<T>* hi) {
+    if constexpr (Tw<T, L>::FULL && L >= 256) return expi_tab<L>(th, hi);
+    else return expi_turns<T>(th);
 }
 
 // v[r] *= W_L^{S r e1} for r = 1..R-1 (R <= 32): table lookups of
@@ -556,30 +609,35 @@ template <typename T, int L> __device__ __forceinline__ cx<T> tw_get(const cx<T>
 template <typename T, int L, int R, int S>
 __device__ __forceinline__ void twiddle_row(cx<T>* v, int e1, const cx<T>* hi, const cx<T>* lo) {
     typedef cx<T> C;
-    C w[8];
-    w[1] = tw_get<T, L>(hi, lo, e1);
-    if constexpr (R > 2) w[2] = tw_get<T, L>(hi, lo, 2 * e1);
-    if constexpr (R > 2) w[3] = cmul(w[1], w[2]);
-    if constexpr (R > 4) {
-        w[4] = tw_get<T, L>(hi, lo, 4 * e1);
-        w[5] = cmul(w[1], w[4]);
-        w[6] = cmul(w[2], w[4]);
-        w[7] = cmul(w[3], w[4]);
-    }
-    C u[4];
-    if constexpr (R > 8) u[1] = tw_get<T, L>(hi, lo, 8 * e1);
-    if constexpr (R > 16) {
-        u[2] = tw_get<T, L>(hi, lo, 16 * e1);
-        u[3] = cmul(u[1], u[2]);
-    }
+    if constexpr (Tw<T, L>::FULL) {
 #pragma unroll
-    for (int r = 1; r < R; ++r) {
-        const int a = r & 7, b = r >> 3;
-        C t;
-        if (b == 0) t = w[a];
-        else if (a == 0) t = u[b];
-        else t = cmul(w[a], u[b]);
-        v[r] = mul_dir<S>(v[r], t);
+        for (int r = 1; r < R; ++r) v[r] = mul_dir<S>(v[r], hi[r * e1]);
+    } else {
+        C w[8];
+        w[1] = tw_get<T, L>(hi, lo, e1);
+        if constexpr (R > 2) w[2] = tw_get<T, L>(hi, lo, 2 * e1);
+        if constexpr (R > 2) w[3] = cmul(w[1], w[2]);
+        if constexpr (R > 4) {
+            w[4] = tw_get<T, L>(hi, lo, 4 * e1);
+            w[5] = cmul(w[1], w[4]);
+            w[6] = cmul(w[2], w[4]);
+            w[7] = cmul(w[3], w[4]);
+        }
+        C u[4];
+        if constexpr (R > 8) u[1] = tw_get<T, L>(hi, lo, 8 * e1);
+        if constexpr (R > 16) {
+            u[2] = tw_get<T, L>(hi, lo, 16 * e1);
+            u[3] = cmul(u[1], u[2]);
+        }
+#pragma unroll
+        for (int r = 1; r < R; ++r) {
+            const int a = r & 7, b = r >> 3;
+            C t;
+            if (b == 0) t = w[a];
+            else if (a == 0) t = u[b];
+            else t = cmul(w[a], u[b]);
+            v[r] = mul_dir<S>(v[r], t);
+        }
     }
 }
 
@@ -784,7 +842,9 @@ template <int KIND> struct Tiling<float, KIND> {
     static constexpr int TE = KIND == 1 ? MPA_KR_TE : MPA_KC_TE;
 };
 template <int KIND> struct Tiling<double, KIND> {
-    static constexpr int E = 16, RMAX = 8, PSH = 3, CMIN = 4, TE = 4096;
+    // radix-16 passes: 1024 points in 29 FP64 instructions an element (16 x
+    // 16 x 4), 41 with radix 8 (8 x 8 x 8 x 2 and two-level twiddle tables)
+    static constexpr int E = 16, RMAX = 16, PSH = 4, CMIN = 4, TE = 4096;
 };
 
 }  // namespace mpa

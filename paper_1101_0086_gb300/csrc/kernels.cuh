@@ -115,7 +115,7 @@ template <typename T, int L> struct KCGeom {
     static constexpr int OSH = 5;  // outer-factor two-level split of n2
     static constexpr int OLO = L < 32 ? L : 32;
     static constexpr int OHI = L > 32 ? L / 32 : 1;
-    static constexpr size_t smem_elems = (size_t)TE + (TE >> P::PSH) + 1 + TwDims<L>::NLO + TwDims<L>::NHI +
+    static constexpr size_t smem_elems = (size_t)TE + (TE >> P::PSH) + 1 + Tw<T, L>::N +
                                          (size_t)G * (OLO + OHI);
     // FP32: + the exp(2 pi i m/1024) table of the per-element phases
     static constexpr size_t smem_bytes = smem_elems * sizeof(cx<T>);
@@ -129,7 +129,7 @@ template <typename T, int L> struct KRGeom {
     static constexpr int OSH = 7;  // outer-factor split of k1
     static constexpr int OLO = L < 128 ? L : 128;
     static constexpr int OHI = L > 128 ? L / 128 : 1;
-    static constexpr size_t smem_elems = (size_t)TE + (TE >> P::PSH) + 1 + TwDims<L>::NLO + TwDims<L>::NHI +
+    static constexpr size_t smem_elems = (size_t)TE + (TE >> P::PSH) + 1 + Tw<T, L>::N +
                                          (size_t)G * (OLO + OHI);
     static constexpr size_t smem_bytes = smem_elems * sizeof(cx<T>);
 };
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(KCGeom<T, L>::NT, KCGeom<T, L>::NT <= 256 ? MP
     C* s = reinterpret_cast<C*>(smem_raw);
     C* thi = s + TE + (TE >> P::PSH) + 1;
     C* tlo = thi + TwDims<L>::NHI;
-    C* olo = tlo + TwDims<L>::NLO;  // [OLO][G]
+    C* olo = thi + Tw<T, L>::N;  // [OLO][G]
     C* ohi = olo + G * Gm::OLO;     // [OHI][G]
     const int tid = threadIdx.x;
     const long long col0 = (long long)blockIdx.x * G;
@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(KCGeom<T, L>::NT, KCGeom<T, L>::NT <= 256 ? MP
                 // MPA step 2: A_hat_j = psi_j exp(i beta(w, z_j) + int G)
                 C ph;
                 if constexpr (FAST) ph = expi_turns_poly(th[r]);
-                else ph = expi_turns<T>(phase_q64(signed_k(c + (long long)row * p.N1, p.N), nc));
+                else ph = expi_at<T, L>(phase_q64(signed_k(c + (long long)row * p.N1, p.N), nc), thi);
                 v = cscale(cmul(v, ph), (T)nc.pre);
             }
             vin[q][r] = v;
@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(KCGeom<T, L>::NT, KCGeom<T, L>::NT <= 256 ? MP
                 const int row = j + r * (L / XF::RL);
                 C ph;
                 if constexpr (FAST) ph = expi_turns_poly(th[r]);
-                else ph = expi_turns<T>(phase_q64(signed_k(c + (long long)row * p.N1, p.N), p.flow));
+                else ph = expi_at<T, L>(phase_q64(signed_k(c + (long long)row * p.N1, p.N), p.flow), thi);
                 vm[q][r] = cscale(cmul(vm[q][r], ph), (T)p.flow.pre);
             }
         }
@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(KCGeom<T, L>::NT, KCGeom<T, L>::NT <= 256 ? MP
                 // V_j = sigma(z_j) dz F[|A_j|^2 A_j] exp(-i beta(w, z_j) - int G)   (Eq. (6))
                 C ph;
                 if constexpr (FAST) ph = expi_turns_poly(th[r]);
-                else ph = expi_turns<T>(phase_q64(signed_k(c + (long long)row * p.N1, p.N), nc));
+                else ph = expi_at<T, L>(phase_q64(signed_k(c + (long long)row * p.N1, p.N), nc), thi);
                 v = cscale(cmul(v, cconj(ph)), (T)nc.post);
             }
             if (MPA_DBG_OK(p.dbg, dst + (long long)row * p.N1, sizeof(C))) dst[(long long)row * p.N1] = v;
@@ -376,7 +376,7 @@ __global__ void __launch_bounds__(KRGeom<T, L>::NT, KRGeom<T, L>::NT <= 256 ? MP
     C* s = reinterpret_cast<C*>(smem_raw);
     C* thi = s + TE + (TE >> P::PSH) + 1;
     C* tlo = thi + TwDims<L>::NHI;
-    C* olo = tlo + TwDims<L>::NLO;  // [G][OLO]
+    C* olo = thi + Tw<T, L>::N;  // [G][OLO]
     C* ohi = olo + G * Gm::OLO;     // [G][OHI]
     const int tid = threadIdx.x;
     const long long row0 = (long long)blockIdx.x * G;
@@ -515,7 +515,7 @@ template <typename T, int L> struct KNGeom {
     static constexpr int G = R::G, TE = R::TE, NT = R::NT;
     typedef Tiling<T, 1> P;
     static constexpr size_t smem_bytes =
-        ((size_t)TE + (TE >> P::PSH) + 1 + TwDims<L>::NLO + TwDims<L>::NHI) * sizeof(cx<T>);
+        ((size_t)TE + (TE >> P::PSH) + 1 + Tw<T, L>::N) * sizeof(cx<T>);
 };
 
 // The node rows row0 .. row0 + G - 1 of a launch (one tile) through steps
@@ -568,7 +568,7 @@ __device__ __forceinline__ void kn_tile(const KNParams<T>& p, long long row0, un
             C v = ok && MPA_DBG_OK(p.dbg, src + k, sizeof(C)) ? ldx<CG>(src + k) : mkc(T(0), T(0));
             C ph;
             if constexpr (FAST) ph = expi_turns_poly(th[r]);
-            else ph = expi_turns<T>(phase_q64(signed_k(k, L), nc));
+            else ph = expi_at<T, L>(phase_q64(signed_k(k, L), nc), thi);
             vin[q][r] = cscale(cmul(v, ph), (T)nc.pre);
         }
     }
@@ -615,7 +615,7 @@ __device__ __forceinline__ void kn_tile(const KNParams<T>& p, long long row0, un
             const int k = j + r * (L / XF::RL);
             C ph;
             if constexpr (FAST) ph = expi_turns_poly(th[r]);
-            else ph = expi_turns<T>(phase_q64(signed_k(k, L), nc));
+            else ph = expi_at<T, L>(phase_q64(signed_k(k, L), nc), thi);
             if (MPA_DBG_OK(p.dbg, dst + k, sizeof(C))) dst[k] = cscale(cmul(vout[q][r], cconj(ph)), (T)nc.post);
         }
     }
