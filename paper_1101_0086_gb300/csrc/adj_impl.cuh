@@ -110,13 +110,13 @@ cudaError_t krk_any(int logL, const KRParams<T>& p, cudaStream_t st) {
     return cudaErrorInvalidValue;
 }
 
-template <typename T, int L, int MODE>
+template <typename T, int L, int MODE, int F>
 cudaError_t ssc_one(const SSCParams<T>& p, cudaStream_t st) {
     if (const cudaError_t eg = launch_gate()) return eg;
-    typedef KCGeom<T, L> Gm;
+    typedef KCGeom<T, L, F> Gm;
     static AttrOnce once;
     const cudaError_t ea = attrs_once(once, [] {
-        cudaError_t e = cudaFuncSetAttribute(ssc_kernel<T, L, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(ssc_kernel<T, L, MODE, F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)Gm::smem_bytes);
         if (e != cudaSuccess) return e;
         return cudaSuccess;
@@ -125,19 +125,19 @@ cudaError_t ssc_one(const SSCParams<T>& p, cudaStream_t st) {
     if (p.N1 % Gm::G != 0) return cudaErrorInvalidValue;
     const bool prof = g_prof_on.load(std::memory_order_relaxed);
     if (prof) prof_begin(st);
-    ssc_kernel<T, L, MODE><<<(unsigned)(p.N1 / Gm::G), Gm::NT, Gm::smem_bytes, st>>>(p);
+    ssc_kernel<T, L, MODE, F><<<(unsigned)(p.N1 / Gm::G), Gm::NT, Gm::smem_bytes, st>>>(p);
     if (prof) prof_end(PK_KC_ADJ, st, 3.0 * (double)p.N * sizeof(cx<T>));
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError();
 }
 
-template <typename T, int L, int MODE>
+template <typename T, int L, int MODE, int F>
 cudaError_t ssr_one(const SSRParams<T>& p, cudaStream_t st) {
     if (const cudaError_t eg = launch_gate()) return eg;
-    typedef KRGeom<T, L> Gm;
+    typedef KRGeom<T, L, F> Gm;
     static AttrOnce once;
     const cudaError_t ea = attrs_once(once, [] {
-        cudaError_t e = cudaFuncSetAttribute(ssr_kernel<T, L, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(ssr_kernel<T, L, MODE, F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)Gm::smem_bytes);
         if (e != cudaSuccess) return e;
         return cudaSuccess;
@@ -146,19 +146,66 @@ cudaError_t ssr_one(const SSRParams<T>& p, cudaStream_t st) {
     if (p.nrows % Gm::G != 0) return cudaErrorInvalidValue;
     const bool prof = g_prof_on.load(std::memory_order_relaxed);
     if (prof) prof_begin(st);
-    ssr_kernel<T, L, MODE><<<(unsigned)(p.nrows / Gm::G), Gm::NT, Gm::smem_bytes, st>>>(p);
+    ssr_kernel<T, L, MODE, F><<<(unsigned)(p.nrows / Gm::G), Gm::NT, Gm::smem_bytes, st>>>(p);
     if (prof) prof_end(PK_KR_ADJ, st, 3.0 * (double)p.nrows * L * sizeof(cx<T>));
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError();
 }
 
+// the tiles of field_tiles(), as the forward passes
+template <typename T, int L, int MODE> cudaError_t ssc_field(const SSCParams<T>& p, cudaStream_t st) {
+    return field_tiles<T>(L, p.N) == 1 ? ssc_one<T, L, MODE, 1>(p, st) : ssc_one<T, L, MODE, 2>(p, st);
+}
+template <typename T, int L, int MODE> cudaError_t ssr_field(const SSRParams<T>& p, cudaStream_t st) {
+    if constexpr (field_tiles<T>(L, 0) == 0) return ssr_one<T, L, MODE, 0>(p, st);
+    else return field_tiles<T>(L, p.N) == 1 ? ssr_one<T, L, MODE, 1>(p, st) : ssr_one<T, L, MODE, 2>(p, st);
+}
 template <typename T, int L>
 cudaError_t ssc_mode(int mode, const SSCParams<T>& p, cudaStream_t st) {
-    return mode == SS_STORE ? ssc_one<T, L, SS_STORE>(p, st) : ssc_one<T, L, SS_REV>(p, st);
+    return mode == SS_STORE ? ssc_field<T, L, SS_STORE>(p, st) : ssc_field<T, L, SS_REV>(p, st);
 }
 template <typename T, int L>
 cudaError_t ssr_mode(int mode, const SSRParams<T>& p, cudaStream_t st) {
-    return mode == SS_STORE ? ssr_one<T, L, SS_STORE>(p, st) : ssr_one<T, L, SS_REV>(p, st);
+    return mode == SS_STORE ? ssr_field<T, L, SS_STORE>(p, st) : ssr_field<T, L, SS_REV>(p, st);
+}
+// columns per tile of ssc and rows per tile of ssr for a field of N samples
+template <typename T, int L> int ss_cols(long long N) {
+    return field_tiles<T>(L, N) == 1 ? KCGeom<T, L, 1>::G : KCGeom<T, L, 2>::G;
+}
+template <typename T, int L> int ss_rows(long long N) {
+    const int f = field_tiles<T>(L, N);
+    return f == 0 ? KRGeom<T, L>::G : f == 1 ? KRGeom<T, L, 1>::G : KRGeom<T, L, 2>::G;
+}
+template <typename T> int ssc_cols_any(int logL, long long N) {
+    switch (logL) {
+        case 4: return ss_cols<T, 16>(N);
+        case 5: return ss_cols<T, 32>(N);
+        case 6: return ss_cols<T, 64>(N);
+        case 7: return ss_cols<T, 128>(N);
+        case 8: return ss_cols<T, 256>(N);
+        case 9: return ss_cols<T, 512>(N);
+        case 10: return ss_cols<T, 1024>(N);
+        case 11: return ss_cols<T, 2048>(N);
+    }
+    return -1;
+}
+template <typename T> int ssr_rows_any(int logL, long long N) {
+    switch (logL) {
+        case 4: return ss_rows<T, 16>(N);
+        case 5: return ss_rows<T, 32>(N);
+        case 6: return ss_rows<T, 64>(N);
+        case 7: return ss_rows<T, 128>(N);
+        case 8: return ss_rows<T, 256>(N);
+        case 9: return ss_rows<T, 512>(N);
+        case 10: return ss_rows<T, 1024>(N);
+        case 11: return ss_rows<T, 2048>(N);
+        case 12: return ss_rows<T, 4096>(N);
+        case 13: return ss_rows<T, 8192>(N);
+        case 14:
+            if constexpr (sizeof(T) == 4) return ss_rows<T, 16384>(N);
+            break;
+    }
+    return -1;
 }
 
 template <typename T>
@@ -340,4 +387,6 @@ cudaError_t scale_to_state_any(const cx<T>* in, double2* state, double scale, lo
     template <> cudaError_t ssr_launch<T>(int mode, int logL, const SSRParams<T>& p, cudaStream_t st) {        \
         return adj::ssr_any<T>(mode, logL, p, st);                                                             \
     }                                                                                                          \
+    template <> int ssc_tile_cols<T>(int logL, long long N) { return adj::ssc_cols_any<T>(logL, N); }          \
+    template <> int ssr_tile_rows<T>(int logL, long long N) { return adj::ssr_rows_any<T>(logL, N); }          \
     }

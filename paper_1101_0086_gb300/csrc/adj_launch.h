@@ -23,5 +23,8 @@ template <typename T> cudaError_t ssr_launch(int mode, int logL, const SSRParams
 // Tile widths of the reverse passes (columns per column tile, rows per row tile).
 template <typename T> int kca_tile_cols(int logL);
 template <typename T> int kra_tile_rows(int logL);
+// and of the split-step's, for a field of N samples
+template <typename T> int ssc_tile_cols(int logL, long long N);
+template <typename T> int ssr_tile_rows(int logL, long long N);
 
 }  // namespace mpa

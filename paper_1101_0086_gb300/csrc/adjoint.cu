@@ -369,19 +369,23 @@ int check_ws(const AdjLayout& a, void* ws, size_t bytes) {
 
 namespace mpa {
 
-// acc[i] += sum_{t < per} part[i per + t], in order (deterministic).
+// acc[i] += sum_{t < per} part[i per + t], one warp per sum, in a fixed order
+// (deterministic).  One thread per sum took about 40 ns a term (a dependent
+// FP64 add and an L2 read): 20 us for the 512 tiles of a 2^20 row pass.
 __global__ void __launch_bounds__(128) reduce_parts_kernel(const double* __restrict__ part, int per, int n,
                                                            double* __restrict__ acc) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (i >= n) return;
     double s = 0.0;
-    for (int t = 0; t < per; ++t) s += part[(long long)i * per + t];
-    acc[i] += s;
+    for (int t = lane; t < per; t += 32) s += part[(long long)i * per + t];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) acc[i] += s;
 }
 
 cudaError_t reduce_parts_launch(const double* part, int per, int n, double* acc, cudaStream_t st) {
     if (const cudaError_t eg = launch_gate()) return eg;
-    reduce_parts_kernel<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(part, per, n, acc);
+    reduce_parts_kernel<<<(unsigned)((n + 3) / 4), 128, 0, st>>>(part, per, n, acc);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError();
 }

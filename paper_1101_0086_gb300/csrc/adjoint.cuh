@@ -474,11 +474,11 @@ template <typename T> struct SSRParams {
     double* part;
 };
 
-template <typename T, int L, int MODE>
-__global__ void __launch_bounds__(KCGeom<T, L>::NT, KCGeom<T, L>::NT <= 256 && sizeof(T) == 4 ? MPA_ADJ_MINB : 1) ssc_kernel(const SSCParams<T> p) {
+template <typename T, int L, int MODE, int F>
+__global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 256 && sizeof(T) == 4 ? MPA_ADJ_MINB : 1) ssc_kernel(const SSCParams<T> p) {
     typedef cx<T> C;
-    typedef KCGeom<T, L> Gm;
-    typedef Tiling<T> P;
+    typedef KCGeom<T, L, F> Gm;
+    typedef typename Gm::P P;
     constexpr int G = Gm::G, TE = Gm::TE, NT = Gm::NT;
     typedef Xform<T, L, G, NT, P::RMAX, +1, LAYOUT_COL, P::PSH, true> XF;
     typedef Xform<T, L, G, NT, P::RMAX, -1, LAYOUT_COL, P::PSH, false> XI;
@@ -557,11 +557,11 @@ __global__ void __launch_bounds__(KCGeom<T, L>::NT, KCGeom<T, L>::NT <= 256 && s
     }
 }
 
-template <typename T, int L, int MODE>
-__global__ void __launch_bounds__(KRGeom<T, L>::NT, KRGeom<T, L>::NT <= 256 && sizeof(T) == 4 ? MPA_ADJ_MINB_R : 1) ssr_kernel(const SSRParams<T> p) {
+template <typename T, int L, int MODE, int F>
+__global__ void __launch_bounds__(KRGeom<T, L, F>::NT, KRGeom<T, L, F>::NT <= 256 && sizeof(T) == 4 ? MPA_ADJ_MINB_R : 1) ssr_kernel(const SSRParams<T> p) {
     typedef cx<T> C;
-    typedef KRGeom<T, L> Gm;
-    typedef Tiling<T, 1> P;
+    typedef KRGeom<T, L, F> Gm;
+    typedef typename Gm::P P;
     constexpr int G = Gm::G, TE = Gm::TE, NT = Gm::NT;
     typedef Xform<T, L, G, NT, P::RMAX, -1, LAYOUT_ROW, P::PSH, false> XI;
     typedef Xform<T, L, G, NT, P::RMAX, +1, LAYOUT_ROW, P::PSH, true> XF;

@@ -830,7 +830,34 @@ template <typename T, int L, int G, int NT, int RMAX, int S, int LAYOUT, int PSH
 #define MPA_KCW_E 16
 #endif
 // KIND 2 = wavefront column pass.
+// KIND 3, 4 = both passes over a single field (transforms, split steps), whose
+// few large tiles would leave SMs idle: fine and medium tiles.
 template <typename T, int KIND = 0> struct Tiling;
+template <> struct Tiling<float, 3> {
+    static constexpr int E = 8, RMAX = 8, PSH = 3, CMIN = 4, TE = 1024;
+};
+template <> struct Tiling<float, 4> {
+    static constexpr int E = 16, RMAX = 16, PSH = 4, CMIN = 4, TE = 1024;
+};
+template <> struct Tiling<double, 3> {
+    static constexpr int E = 4, RMAX = 4, PSH = 2, CMIN = 1, TE = 256;
+};
+template <> struct Tiling<double, 4> {
+    static constexpr int E = 8, RMAX = 8, PSH = 3, CMIN = 1, TE = 256;
+};
+// The tiles of a single-field pass of length L over `elems` elements: 0 the
+// large tiles of the MPA passes, 1 fine, 2 medium.  Measured, us a split step
+// (both passes), large / medium / fine.  FP32 (launches and latency, then
+// warps to hide it): 2^12 30.7 / 16.0 / 11.9, 2^18 26.4 / 18.2 / 13.8, 2^19
+// 26.3 / 18.0 / 18.1, 2^20 28.8 / 23.2 / 28.6, 2^22 74.3 / 71.0 / 97.4.  FP64
+// (an FP64 instruction occupies one of an SM's four schedulers for 76 clocks,
+// so small fields need their elements spread over all of them): 2^12 244 / 71
+// / 46, 2^16 228 / 69 / 42, 2^17 221 / 70.6 / 68.4, 2^18 230 / 123 / 128, 2^20
+// 443 / 421 / 425, 2^22 1709 / 1691 / 1835.  Rows above 2048 points keep the
+// large tiles (one or a few rows each).
+template <typename T> __host__ __device__ constexpr int field_tiles(int L, long long elems) {
+    return L > 2048 ? 0 : elems <= (sizeof(T) == 8 ? 1ll << 16 : 1ll << 18) ? 1 : 2;
+}
 #ifndef MPA_RMAX32
 #define MPA_RMAX32 32
 #endif

@@ -3,19 +3,19 @@
 
 namespace mpa {
 
-template <int L, int MODE>
+template <int L, int MODE, int F = 0>
 static cudaError_t kc_one(const KCParams<double>& pin, cudaStream_t st) {
     if (const cudaError_t eg = launch_gate()) return eg;
     // callers that leave the link fields unset launch one run of nodes
     KCParams<double> p = pin;
     if (p.npl <= 0) p.npl = (int)(p.ncols >> p.logN1) > 0 ? (int)(p.ncols >> p.logN1) : 1;
-    typedef KCGeom<double, L> Gm;
+    typedef KCGeom<double, L, F> Gm;
     static AttrOnce once;
     const cudaError_t ea = attrs_once(once, [] {
-        cudaError_t e = cudaFuncSetAttribute(kc_kernel<double, L, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(kc_kernel<double, L, MODE, F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)Gm::smem_bytes);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(kc_kernel<double, L, MODE>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        e = cudaFuncSetAttribute(kc_kernel<double, L, MODE, F>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
         if (e != cudaSuccess) return e;
         return cudaSuccess;
     });
@@ -24,7 +24,7 @@ static cudaError_t kc_one(const KCParams<double>& pin, cudaStream_t st) {
     if (nblk <= 0) return cudaSuccess;
     const bool prof = g_prof_on.load(std::memory_order_relaxed);
     if (prof) prof_begin(st);
-    kc_kernel<double, L, MODE><<<(unsigned)nblk, Gm::NT, Gm::smem_bytes, st>>>(p);
+    kc_kernel<double, L, MODE, F><<<(unsigned)nblk, Gm::NT, Gm::smem_bytes, st>>>(p);
     if (prof) {
         // algorithmic bytes: every tile element read once and written once
         // (a shared source, src_stride == 0, is read once for all nodes)
@@ -36,14 +36,19 @@ static cudaError_t kc_one(const KCParams<double>& pin, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+template <int L, int MODE> static cudaError_t kc_field(const KCParams<double>& p, cudaStream_t st) {
+    return field_tiles<double>(L, p.ncols * L) == 1 ? kc_one<L, MODE, 1>(p, st) : kc_one<L, MODE, 2>(p, st);
+}
+
 template <int L>
 static cudaError_t kc_mode(int mode, const KCParams<double>& p, cudaStream_t st) {
+    // passes of the MPA levels (error word) are many nodes: large tiles
     switch (mode) {
         case KC_MPA_PRE: return kc_one<L, KC_MPA_PRE>(p, st);
         case KC_MPA_POST: return kc_one<L, KC_MPA_POST>(p, st);
-        case KC_SS_STEP: return kc_one<L, KC_SS_STEP>(p, st);
-        case KC_FWD: return kc_one<L, KC_FWD>(p, st);
-        case KC_INV: return kc_one<L, KC_INV>(p, st);
+        case KC_SS_STEP: return kc_field<L, KC_SS_STEP>(p, st);
+        case KC_FWD: return p.err ? kc_one<L, KC_FWD>(p, st) : kc_field<L, KC_FWD>(p, st);
+        case KC_INV: return p.err ? kc_one<L, KC_INV>(p, st) : kc_field<L, KC_INV>(p, st);
     }
     return cudaErrorInvalidValue;
 }

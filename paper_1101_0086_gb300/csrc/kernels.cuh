@@ -107,8 +107,9 @@ template <typename T> struct KRParams {
 };
 
 // Column pass geometry for column length L: G columns per tile, NT threads.
-template <typename T, int L> struct KCGeom {
-    typedef Tiling<T> P;
+// F: the tiles of field_tiles().
+template <typename T, int L, int F = 0> struct KCGeom {
+    typedef Tiling<T, F ? F + 2 : 0> P;
     static constexpr int G = (P::TE / L) > P::CMIN ? (P::TE / L) : P::CMIN;
     static constexpr int TE = G * L;
     static constexpr int NT = TE / P::E;
@@ -121,8 +122,8 @@ template <typename T, int L> struct KCGeom {
     static constexpr size_t smem_bytes = smem_elems * sizeof(cx<T>);
 };
 
-template <typename T, int L> struct KRGeom {
-    typedef Tiling<T, 1> P;
+template <typename T, int L, int F = 0> struct KRGeom {
+    typedef Tiling<T, F ? F + 2 : 1> P;
     static constexpr int G = (P::TE / L) > 1 ? (P::TE / L) : 1;
     static constexpr int TE = G * L;
     static constexpr int NT = TE / P::E;
@@ -180,12 +181,12 @@ __device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
 #ifndef MPA_KR_MINB
 #define MPA_KR_MINB 2
 #endif
-template <typename T, int L, int MODE>
-__global__ void __launch_bounds__(KCGeom<T, L>::NT, KCGeom<T, L>::NT <= 256 ? MPA_KC_MINB : 1)
+template <typename T, int L, int MODE, int F = 0>
+__global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 256 ? MPA_KC_MINB : 1)
     kc_kernel(const KCParams<T> p) {
     typedef cx<T> C;
-    typedef KCGeom<T, L> Gm;
-    typedef Tiling<T> P;
+    typedef KCGeom<T, L, F> Gm;
+    typedef typename Gm::P P;
     constexpr int G = Gm::G, TE = Gm::TE, NT = Gm::NT;
     constexpr bool FWD = (MODE == KC_MPA_POST || MODE == KC_SS_STEP || MODE == KC_FWD);
     constexpr bool INV = (MODE == KC_MPA_PRE || MODE == KC_SS_STEP || MODE == KC_INV);
@@ -357,12 +358,12 @@ __global__ void __launch_bounds__(KCGeom<T, L>::NT, KCGeom<T, L>::NT <= 256 ? MP
     }
 }
 
-template <typename T, int L, int MODE>
-__global__ void __launch_bounds__(KRGeom<T, L>::NT, KRGeom<T, L>::NT <= 256 ? MPA_KR_MINB : 1)
+template <typename T, int L, int MODE, int F = 0>
+__global__ void __launch_bounds__(KRGeom<T, L, F>::NT, KRGeom<T, L, F>::NT <= 256 ? MPA_KR_MINB : 1)
     kr_kernel(const KRParams<T> p) {
     typedef cx<T> C;
-    typedef KRGeom<T, L> Gm;
-    typedef Tiling<T, 1> P;
+    typedef KRGeom<T, L, F> Gm;
+    typedef typename Gm::P P;
     constexpr int G = Gm::G, TE = Gm::TE, NT = Gm::NT;
     constexpr bool INV = (MODE != KR_FWD);
     constexpr bool FWD = (MODE != KR_INV);
@@ -406,7 +407,7 @@ __global__ void __launch_bounds__(KRGeom<T, L>::NT, KRGeom<T, L>::NT <= 256 ? MP
                                                                                      : mkc(T(0), T(0));
     }
 
-    if constexpr (sizeof(T) == 4 && MPA_L2PF_KR > 0) {
+    if constexpr (F == 0 && sizeof(T) == 4 && MPA_L2PF_KR > 0) {
         const long long tb = (long long)blockIdx.x + MPA_L2PF_KR;
         const long long r0 = tb * G;
         if (tb < (long long)gridDim.x && r0 < p.nrows) {

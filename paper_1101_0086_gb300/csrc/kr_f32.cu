@@ -46,16 +46,16 @@ bool kr_staged(int mode, int logL, const KRParams<float>& p) {
     return MPA_KR_STAGED && p.err && (mode == KR_MPA || mode == KR_SS) && logL >= 9 && logL <= 13;
 }
 
-template <int L, int MODE>
+template <int L, int MODE, int F = 0>
 static cudaError_t kr_one(const KRParams<float>& p, cudaStream_t st) {
     if (const cudaError_t eg = launch_gate()) return eg;
-    typedef KRGeom<float, L> Gm;
+    typedef KRGeom<float, L, F> Gm;
     static AttrOnce once;
     const cudaError_t ea = attrs_once(once, [] {
-        cudaError_t e = cudaFuncSetAttribute(kr_kernel<float, L, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(kr_kernel<float, L, MODE, F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)Gm::smem_bytes);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(kr_kernel<float, L, MODE>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        e = cudaFuncSetAttribute(kr_kernel<float, L, MODE, F>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
         if (e != cudaSuccess) return e;
         return cudaSuccess;
     });
@@ -64,19 +64,24 @@ static cudaError_t kr_one(const KRParams<float>& p, cudaStream_t st) {
     if (nblk <= 0) return cudaSuccess;
     const bool prof = g_prof_on.load(std::memory_order_relaxed);
     if (prof) prof_begin(st);
-    kr_kernel<float, L, MODE><<<(unsigned)nblk, Gm::NT, Gm::smem_bytes, st>>>(p);
+    kr_kernel<float, L, MODE, F><<<(unsigned)nblk, Gm::NT, Gm::smem_bytes, st>>>(p);
     if (prof) prof_end(prof_kr_kind(MODE), st, 2.0 * (double)p.nrows * L * sizeof(cx<float>));
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError();
+}
+
+template <int L, int MODE> static cudaError_t kr_field(const KRParams<float>& p, cudaStream_t st) {
+    if constexpr (field_tiles<float>(L, 0) == 0) return kr_one<L, MODE>(p, st);
+    else return field_tiles<float>(L, p.nrows * L) == 1 ? kr_one<L, MODE, 1>(p, st) : kr_one<L, MODE, 2>(p, st);
 }
 
 template <int L>
 static cudaError_t kr_mode(int mode, const KRParams<float>& p, cudaStream_t st) {
     switch (mode) {
         case KR_MPA: return kr_one<L, KR_MPA>(p, st);
-        case KR_SS: return kr_one<L, KR_SS>(p, st);
-        case KR_FWD: return kr_one<L, KR_FWD>(p, st);
-        case KR_INV: return kr_one<L, KR_INV>(p, st);
+        case KR_SS: return kr_field<L, KR_SS>(p, st);
+        case KR_FWD: return kr_field<L, KR_FWD>(p, st);
+        case KR_INV: return kr_field<L, KR_INV>(p, st);
     }
     return cudaErrorInvalidValue;
 }

@@ -42,8 +42,8 @@ int ss_layout(const HostMap& m, const Split& s, int prec, double dz, double z_fr
     if (a->Kc > a->K) a->Kc = a->K;
     a->n_ck = (a->K + a->Kc - 1) / a->Kc;
     const bool f32 = prec == MPA_FP32;
-    const int gc = f32 ? kca_tile_cols<float>(s.logN2) : kca_tile_cols<double>(s.logN2);
-    const int gr = f32 ? kra_tile_rows<float>(s.logN1) : kra_tile_rows<double>(s.logN1);
+    const int gc = f32 ? ssc_tile_cols<float>(s.logN2, s.N) : ssc_tile_cols<double>(s.logN2, s.N);
+    const int gr = f32 ? ssr_tile_rows<float>(s.logN1, s.N) : ssr_tile_rows<double>(s.logN1, s.N);
     if (gc <= 0 || gr <= 0 || gc > s.N1 || gr > s.N2) return MPA_ERR_UNSUPPORTED_N;
     a->tiles_c = s.N1 / gc;
     a->tiles_r = s.N2 / gr;

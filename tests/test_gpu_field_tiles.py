@@ -1,4 +1,5 @@
-"""FP64 transforms, split-steps and node transforms with full twiddle tables
+"""Transforms and split-steps of single fields on their fine and medium tiles,
+and FP64 node transforms, with full twiddle tables
 (lengths up to 2048, phases from the table from 256 on) at every length of
 rows and columns, against the oracle.
 
@@ -59,3 +60,29 @@ def test_fp64_interval(M, logn, split):
     plan.propagate(d, 45.0, 50.0)
     assert plan.status_code() == 0
     assert oracle.rel_l2(d.cpu().numpy(), oracle.mpa(a, dm_map(1), T, 45.0, 50.0, 5.0, 6, 2)) < 1e-12
+
+
+@pytest.mark.parametrize("logn", [8, 10, 13, 16, 18, 19, 20, 22])
+def test_fp32_transform_pair(M, logn):
+    """Fine and medium tiles in FP32: 22 roundings at 6e-8 and their partial
+    sums' growth, 4e-6."""
+    import torch
+    a = random_field(1 << logn, logn).astype(np.complex64)
+    d = torch.from_numpy(a).cuda()
+    M.fft(d, +1)
+    assert oracle.rel_l2(d.cpu().numpy(), oracle.fft(a.astype(np.complex128), +1)) < 4e-6
+    M.fft(d, -1)
+    assert oracle.rel_l2(d.cpu().numpy(), a) < 4e-6
+
+
+@pytest.mark.parametrize("logn", [9, 14, 18, 19, 21])
+def test_fp32_split_step(M, logn):
+    """Eight steps of two transforms: 16 x 22 roundings at 6e-8, 2e-5."""
+    import torch
+    n, spp = 1 << logn, 64 if logn < 14 else 128
+    T = 100.0 * n / spp
+    a = wdm_field(n, T, 4, 50.0, n // spp, 30.0, 2.0, "qpsk", seed=logn).astype(np.complex64)
+    d = torch.from_numpy(a).cuda()
+    M.ss_propagate(d, dm_map(1), T, 0.05, 44.8, 45.2)
+    ref = oracle.ss(a.astype(np.complex128), dm_map(1), T, 44.8, 45.2, 0.05)
+    assert oracle.rel_l2(d.cpu().numpy(), ref) < 2e-5
