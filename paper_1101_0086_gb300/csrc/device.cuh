@@ -641,12 +641,36 @@ __device__ __forceinline__ void twiddle_row(cx<T>* v, int e1, const cx<T>* hi, c
     }
 }
 
+// Direct twiddle table of a pass (FP32): W_{NS R}^{r k}, r < R, k < NS, laid
+// out as [r / 2][k][r mod 2], so that a thread reads its R factors as R / 2
+// 16-byte loads at compile-time offsets from its k; neighbouring threads hold
+// neighbouring k (or the same: a broadcast), without bank conflicts.  Against
+// twiddle_row it trades the lookups' products, 21 to 26 of them for R = 32, and
+// their index arithmetic for loads (4.2 instructions an element and pass).
+template <int NS, int R> __device__ __forceinline__ void dt_fill(float2* t, int tid, int nt) {
+    constexpr int LG = TwDims<NS * R>::logL;
+    static_assert((1 << LG) == NS * R, "a power of two");
+    for (int i = tid; i < NS * R; i += nt) {
+        const int k = (i >> 1) % NS, r = 2 * ((i >> 1) / NS) + (i & 1);
+        t[i] = expi_ratio<float>((long long)r * k, LG);
+    }
+}
+template <int NS, int R, int S> __device__ __forceinline__ void dt_row(float2* v, const float2* t, int k) {
+    const float4* q = reinterpret_cast<const float4*>(t) + k;
+#pragma unroll
+    for (int h = 0; h < R / 2; ++h) {
+        const float4 w = q[h * NS];
+        if (h > 0) v[2 * h] = mul_dir<S>(v[2 * h], make_float2(w.x, w.y));
+        v[2 * h + 1] = mul_dir<S>(v[2 * h + 1], make_float2(w.z, w.w));
+    }
+}
+
 // One radix-R Stockham pass over the tile (in place, barrier-separated
 // read and write phases).  Butterfly j of transform g reads elements
 // j + r L/R, applies W_{NS R}^{S r (j mod NS)}, does the R-point DFT and
 // writes to (j - j mod NS) R + j mod NS + r NS.
-template <typename T, int L, int G, int NT, int R, int NS, int S, int LAYOUT, int PSH, bool SF, int GRP = 0>
-__device__ __forceinline__ void stockham_pass(cx<T>* s, const cx<T>* hi, const cx<T>* lo) {
+template <typename T, int L, int G, int NT, int R, int NS, int S, int LAYOUT, int PSH, bool SF, int GRP = 0, bool DT = false>
+__device__ __forceinline__ void stockham_pass(cx<T>* s, const cx<T>* hi, const cx<T>* lo, const cx<T>* dt = nullptr) {
     typedef cx<T> C;
     constexpr int NB = (L / R) * G;
     static_assert(NB % NT == 0, "butterflies must divide among threads");
@@ -666,7 +690,8 @@ __device__ __forceinline__ void stockham_pass(cx<T>* s, const cx<T>* hi, const c
 #pragma unroll
             for (int r = 0; r < R; ++r) v[q][r] = s[phys<PSH>(eidx<LAYOUT, L, G>(j + r * (L / R), g))];
         }
-        if constexpr (NS > 1) twiddle_row<T, L, R, S>(v[q], (j & (NS - 1)) * (L / (NS * R)), hi, lo);
+        if constexpr (DT) dt_row<NS, R, S>(v[q], dt, j & (NS - 1));
+        else if constexpr (NS > 1) twiddle_row<T, L, R, S>(v[q], (j & (NS - 1)) * (L / (NS * R)), hi, lo);
         Dft<R, S, C>::run(v[q]);
     }
     gsync<GRP, NT>();
@@ -710,13 +735,13 @@ template <int L, int RMAX> struct Sched {
     template <bool SF> __host__ __device__ static constexpr int ns(int p) { return p == 0 ? 1 : ns<SF>(p - 1) * radix<SF>(p - 1); }
 };
 
-template <typename T, int L, int G, int NT, int RMAX, int S, int LAYOUT, int PSH, bool SF, int P, int NP, int GRP = 0>
-__device__ __forceinline__ void mid_passes(cx<T>* s, const cx<T>* hi, const cx<T>* lo) {
+template <typename T, int L, int G, int NT, int RMAX, int S, int LAYOUT, int PSH, bool SF, int P, int NP, int GRP, bool DT>
+__device__ __forceinline__ void mid_passes(cx<T>* s, const cx<T>* hi, const cx<T>* lo, const cx<T>* dt) {
     if constexpr (P < NP - 1) {
         typedef Sched<L, RMAX> SC;
-        stockham_pass<T, L, G, NT, SC::template radix<SF>(P), SC::template ns<SF>(P), S, LAYOUT, PSH, SF, GRP>(s, hi,
-                                                                                                              lo);
-        mid_passes<T, L, G, NT, RMAX, S, LAYOUT, PSH, SF, P + 1, NP, GRP>(s, hi, lo);
+        stockham_pass<T, L, G, NT, SC::template radix<SF>(P), SC::template ns<SF>(P), S, LAYOUT, PSH, SF, GRP,
+                      DT && P == 1>(s, hi, lo, dt);
+        mid_passes<T, L, G, NT, RMAX, S, LAYOUT, PSH, SF, P + 1, NP, GRP, DT>(s, hi, lo, dt);
     }
 }
 
@@ -735,8 +760,11 @@ template <int LAYOUT, int L, int G, int R> __host__ __device__ __forceinline__ v
 // j + r L/R0 of butterfly b = tid + q NT (R0 = first radix), vout[q][r]
 // receives output element j + r L/RL (RL = last radix).  Shared memory is
 // used by the middle passes only; the transform ends with a barrier so the
-// caller may reuse `s`.  GRP as for gtid/gsync.
-template <typename T, int L, int G, int NT, int RMAX, int S, int LAYOUT, int PSH, bool SF, int GRP = 0> struct Xform {
+// caller may reuse `s`.  GRP as for gtid/gsync.  USE_DT: the second pass reads
+// its twiddles from a direct table of DTN entries (where that is at most 1024;
+// 0: none) that the caller fills with dt_init and passes to run.
+template <typename T, int L, int G, int NT, int RMAX, int S, int LAYOUT, int PSH, bool SF, int GRP = 0, bool USE_DT = false>
+struct Xform {
     typedef Sched<L, RMAX> SC;
     typedef cx<T> C;
     static constexpr int NP = SC::NP;
@@ -745,19 +773,27 @@ template <typename T, int L, int G, int NT, int RMAX, int S, int LAYOUT, int PSH
     static constexpr int Q0 = (L / R0) * G / NT;
     static constexpr int QL = (L / RL) * G / NT;
     static_assert((L / R0) * G % NT == 0 && (L / RL) * G % NT == 0, "butterflies must divide among threads");
+    static constexpr int NS1 = NP > 1 ? SC::template ns<SF>(NP > 1 ? 1 : 0) : 1;
+    static constexpr int R1 = NP > 1 ? SC::template radix<SF>(NP > 1 ? 1 : 0) : 1;
+    static constexpr int DTN = USE_DT && NP > 1 && NS1 * R1 <= 1024 ? NS1 * R1 : 0;
+    static constexpr bool DT = DTN > 0;
+    static __device__ __forceinline__ void dt_init(C* t, int tid, int nt) {
+        if constexpr (DT) dt_fill<NS1, R1>(t, tid, nt);
+    }
 
     struct NoHook {
         __device__ __forceinline__ void operator()() const {}
     };
-    static __device__ __forceinline__ void run(C (&vin)[Q0][R0], C (&vout)[QL][RL], C* s, const C* hi, const C* lo) {
-        run(vin, vout, s, hi, lo, NoHook());
+    static __device__ __forceinline__ void run(C (&vin)[Q0][R0], C (&vout)[QL][RL], C* s, const C* hi, const C* lo,
+                                               const C* dt = nullptr) {
+        run(vin, vout, s, hi, lo, dt, NoHook());
     }
     // hook() runs once the first pass has left the registers for shared
     // memory (after its barrier; at the start for a single-pass transform),
     // where the caller's own work needs the fewest registers.
     template <class Hook>
     static __device__ __forceinline__ void run(C (&vin)[Q0][R0], C (&vout)[QL][RL], C* s, const C* hi, const C* lo,
-                                               Hook&& hook) {
+                                               const C* dt, Hook&& hook) {
         if constexpr (NP == 1) {
             hook();
 #pragma unroll
@@ -787,7 +823,7 @@ template <typename T, int L, int G, int NT, int RMAX, int S, int LAYOUT, int PSH
             }
             gsync<GRP, NT>();
             hook();
-            mid_passes<T, L, G, NT, RMAX, S, LAYOUT, PSH, SF, 1, NP, GRP>(s, hi, lo);
+            mid_passes<T, L, G, NT, RMAX, S, LAYOUT, PSH, SF, 1, NP, GRP, DT>(s, hi, lo, dt);
             // last pass (NS = L/RL, so k = j): gather j + r L/RL, twiddle W_L^{S r j}, DFT
 #pragma unroll
             for (int q = 0; q < QL; ++q) {
@@ -802,7 +838,8 @@ template <typename T, int L, int G, int NT, int RMAX, int S, int LAYOUT, int PSH
 #pragma unroll
                     for (int r = 0; r < RL; ++r) vout[q][r] = s[phys<PSH>(eidx<LAYOUT, L, G>(j + r * (L / RL), g))];
                 }
-                twiddle_row<T, L, RL, S>(vout[q], j, hi, lo);
+                if constexpr (DT && NP == 2) dt_row<NS1, R1, S>(vout[q], dt, j);
+                else twiddle_row<T, L, RL, S>(vout[q], j, hi, lo);
                 Dft<RL, S, C>::run(vout[q]);
             }
             gsync<GRP, NT>();

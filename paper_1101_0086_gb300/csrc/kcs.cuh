@@ -35,16 +35,25 @@ template <int L> struct KCSTile {
 // mbarriers, four slots of node constants (those of CTA-local tile i in
 // slot i mod 4, copied with the tile), the twiddle tables of both groups,
 // then per group its exchange buffer and outer-factor tables.
+// Direct twiddle tables (dt_fill) in the inverse passes, which multiply
+// second passes of radix 32, 16 and 8 by them (1024 points: 462 -> 442 us a
+// level of 2^20 x 143), and in the forward passes of 256 and 1024 points (128
+// -> 102 us at 2^18, 411 -> 402 us at 2^20); the forward pass of 512 points is
+// slower with one (104 -> 115 us at 2^18).
 template <int L> struct KCSGeom {
     typedef KCSTile<L> Gm;
     typedef Tiling<float> P;
+    typedef Xform<float, L, Gm::G, Gm::NT, P::RMAX, +1, LAYOUT_COL, P::PSH, true, 1, L == 256 || L == 1024> XF;
+    typedef Xform<float, L, Gm::G, Gm::NT, P::RMAX, -1, LAYOUT_COL, P::PSH, false, 1, true> XI;
+    static constexpr int DTN = XF::DTN > XI::DTN ? XF::DTN : XI::DTN;
     static constexpr size_t al(size_t x) { return (x + 127) & ~(size_t)127; }
     static constexpr size_t STAGE_BYTES = (size_t)Gm::TE * sizeof(float2);
     static constexpr size_t BAR_OFF = STAGE_BYTES;
     static constexpr size_t NODE_OFF = BAR_OFF + 16;  // 4 NodeC slots: tile i's node constants in slot i mod 4
     static constexpr size_t TW_OFF = BAR_OFF + 256;
     static_assert(sizeof(NodeC) == 48 && 16 + 4 * sizeof(NodeC) <= 256, "node-constant slots");
-    static constexpr size_t GRP_OFF = al(TW_OFF + (size_t)(TwDims<L>::NLO + TwDims<L>::NHI) * sizeof(float2));
+    static constexpr size_t DT_OFF = al(TW_OFF + (size_t)(TwDims<L>::NLO + TwDims<L>::NHI) * sizeof(float2));
+    static constexpr size_t GRP_OFF = al(DT_OFF + (size_t)DTN * sizeof(float2));
     static constexpr size_t S_ELEMS = (size_t)Gm::TE + (Gm::TE >> P::PSH) + 1;
     static constexpr size_t GRP_BYTES = al((S_ELEMS + (size_t)Gm::G * (Gm::OLO + Gm::OHI)) * sizeof(float2));
     static constexpr size_t smem_bytes = GRP_OFF + 2 * GRP_BYTES;
@@ -147,9 +156,7 @@ __global__ void __launch_bounds__(KCSGeom<L>::THREADS, 1)
     typedef Tiling<float> P;
     constexpr int G = Gm::G, NT = Gm::NT;
     constexpr bool INV = MODE != KC_FWD, PRE = MODE == KC_MPA_PRE;
-    typedef Xform<float, L, G, NT, P::RMAX, +1, LAYOUT_COL, P::PSH, true, 1> XF;
-    typedef Xform<float, L, G, NT, P::RMAX, -1, LAYOUT_COL, P::PSH, false, 1> XI;
-    typedef typename std::conditional<INV, XI, XF>::type XA;
+    typedef typename std::conditional<INV, typename SG::XI, typename SG::XF>::type XA;
     extern __shared__ __align__(128) unsigned char smem_staged[];
     C* stage = reinterpret_cast<C*>(smem_staged);
     unsigned long long* bar = reinterpret_cast<unsigned long long*>(smem_staged + SG::BAR_OFF);
@@ -169,6 +176,8 @@ __global__ void __launch_bounds__(KCSGeom<L>::THREADS, 1)
         mbar_init_fence();
     }
     tw_init<float, L>(thi, tlo, (int)threadIdx.x, SG::THREADS);
+    C* dt = reinterpret_cast<C*>(smem_staged + SG::DT_OFF);
+    XA::dt_init(dt, (int)threadIdx.x, SG::THREADS);
     __syncthreads();
     // the first tile is copied by group 1 (whose own first tile comes later)
     if (grp == 1 && (int)blockIdx.x < ntiles) kcs_fetch<L, PRE>(p, blockIdx.x, stage, &nslot[0], &bar[0], tid);
@@ -246,7 +255,7 @@ __global__ void __launch_bounds__(KCSGeom<L>::THREADS, 1)
         if constexpr (!LATE) fetch_next();
         constexpr int QO = XA::QL, RO = XA::RL;
         C vout[QO][RO];
-        XA::run(vin, vout, s, thi, tlo, [&] {
+        XA::run(vin, vout, s, thi, tlo, dt, [&] {
             if constexpr (LATE) fetch_next();
         });
 

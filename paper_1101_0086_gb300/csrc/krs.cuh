@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(KRSGeom<L>::THREADS, 1) krs_kernel(const KRPar
         }
         C vm[XI::QL][XI::RL];
         // the next tile's copy starts once the first pass has left the registers
-        XI::run(vin, vm, s, thi, tlo, [&] {
+        XI::run(vin, vm, s, thi, tlo, nullptr, [&] {
             const int tn = t + (int)gridDim.x;
             if (tid == 0 && tn < ntiles) {
                 fence_proxy_async_smem();
