@@ -495,6 +495,7 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
     const int N1m = p.N1 - 1;
     constexpr bool FAST = sizeof(T) == 4;
 
+    pdl_go();
     tw_init<T, L>(thi, tlo, tid, NT);
     for (int i = tid; i < G * (Gm::OLO + Gm::OHI); i += NT) {
         const int g = i % G, m = i / G;
@@ -503,6 +504,7 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
         else ohi[(m - Gm::OLO) * G + g] = expi_ratio<T>(-k1 * ((long long)(m - Gm::OLO) << Gm::OSH), p.logN);
     }
     __syncthreads();
+    pdl_wait();
 
     C vin[XF::Q0][XF::R0];
 #pragma unroll
@@ -576,6 +578,7 @@ __global__ void __launch_bounds__(KRGeom<T, L, F>::NT, KRGeom<T, L, F>::NT <= 25
     const int tid = threadIdx.x;
     const long long row0 = (long long)blockIdx.x * G;
 
+    pdl_go();
     tw_init<T, L>(thi, tlo, tid, NT);
     for (int i = tid; i < G * (Gm::OLO + Gm::OHI); i += NT) {
         const int g = i / (Gm::OLO + Gm::OHI), m = i % (Gm::OLO + Gm::OHI);
@@ -584,6 +587,7 @@ __global__ void __launch_bounds__(KRGeom<T, L, F>::NT, KRGeom<T, L, F>::NT <= 25
         else ohi[g * Gm::OHI + (m - Gm::OLO)] = expi_ratio<T>(n2 * ((long long)(m - Gm::OLO) << Gm::OSH), p.logN);
     }
     __syncthreads();
+    pdl_wait();
 
     C vin[XI::Q0][XI::R0];
 #pragma unroll

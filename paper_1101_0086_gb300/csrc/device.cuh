@@ -435,6 +435,20 @@ template <typename T> __device__ __forceinline__ cx<T> expi_ratio(long long e, i
     return mkc(c, s);
 }
 
+// ------------------------------------------------- dependent launches
+// A kernel launched with launch_pdl (launch.h) may start while the kernel
+// before it in its stream still runs: it prepares what needs no memory (its
+// twiddle tables), then pdl_wait() returns once every earlier kernel of the
+// stream has completed and its writes are visible.  pdl_go() lets the next
+// kernel start in the same way as soon as every block of this one has called
+// it.  Every global access comes after pdl_wait().  Both do nothing in a
+// kernel launched without the attribute.  Kernels that a scan follows call
+// pdl_go() at their end: a scan of a few blocks that starts while most SMs are
+// still busy is packed onto the first free ones (2^14 x 801 nodes: 72 -> 108
+// us).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ------------------------------------------------- thread groups
 // A transform runs on the whole block (GRP = 0: threadIdx.x, __syncthreads)
 // or on one of several NT-thread groups of the block (GRP = 1: the thread's

@@ -32,14 +32,14 @@ static cudaError_t kcs_one(const KCParams<float>& p, cudaStream_t st) {
     const unsigned grid = (unsigned)(ntiles < sms ? ntiles : sms);  // one CTA per SM
     const bool prof = g_prof_on.load(std::memory_order_relaxed);
     if (prof) prof_begin(st);
-    kcs_kernel<L, MODE><<<grid, SG::THREADS, SG::smem_bytes, st>>>(p);
+    const cudaError_t el = launch_pdl(true, kcs_kernel<L, MODE>, grid, SG::THREADS, SG::smem_bytes, st, p);
     if (prof) {
         const double cs = (double)sizeof(cx<float>), tile = (double)p.ncols * L;
         const double rd = p.src_stride == 0 ? (double)p.ncols / p.npl * L : tile;
         prof_end(prof_kc_kind(MODE, p.err != nullptr), st, (rd + tile) * cs);
     }
     g_launches.fetch_add(1, std::memory_order_relaxed);
-    return cudaGetLastError();
+    return el;
 }
 
 static constexpr int ilog2_const(int x) { return x <= 1 ? 0 : 1 + ilog2_const(x / 2); }
@@ -99,7 +99,7 @@ static cudaError_t kc_one(const KCParams<float>& pin, cudaStream_t st) {
     if (nblk <= 0) return cudaSuccess;
     const bool prof = g_prof_on.load(std::memory_order_relaxed);
     if (prof) prof_begin(st);
-    kc_kernel<float, L, MODE, F><<<(unsigned)nblk, Gm::NT, Gm::smem_bytes, st>>>(p);
+    const cudaError_t el = launch_pdl(true, kc_kernel<float, L, MODE, F>, (unsigned)nblk, Gm::NT, Gm::smem_bytes, st, p);
     if (prof) {
         // algorithmic bytes: every tile element read once and written once
         // (a shared source, src_stride == 0, is read once for all nodes)
@@ -108,7 +108,7 @@ static cudaError_t kc_one(const KCParams<float>& pin, cudaStream_t st) {
         prof_end(prof_kc_kind(MODE, p.err != nullptr), st, (rd + tile) * cs);
     }
     g_launches.fetch_add(1, std::memory_order_relaxed);
-    return cudaGetLastError();
+    return el;
 }
 
 template <int L, int MODE> static cudaError_t kc_field(const KCParams<float>& p, cudaStream_t st) {

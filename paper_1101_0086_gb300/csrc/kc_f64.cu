@@ -24,7 +24,7 @@ static cudaError_t kc_one(const KCParams<double>& pin, cudaStream_t st) {
     if (nblk <= 0) return cudaSuccess;
     const bool prof = g_prof_on.load(std::memory_order_relaxed);
     if (prof) prof_begin(st);
-    kc_kernel<double, L, MODE, F><<<(unsigned)nblk, Gm::NT, Gm::smem_bytes, st>>>(p);
+    const cudaError_t el = launch_pdl(F == 0 || pdl_field<double>(p.N), kc_kernel<double, L, MODE, F>, (unsigned)nblk, Gm::NT, Gm::smem_bytes, st, p);
     if (prof) {
         // algorithmic bytes: every tile element read once and written once
         // (a shared source, src_stride == 0, is read once for all nodes)
@@ -33,7 +33,7 @@ static cudaError_t kc_one(const KCParams<double>& pin, cudaStream_t st) {
         prof_end(prof_kc_kind(MODE, p.err != nullptr), st, (rd + tile) * cs);
     }
     g_launches.fetch_add(1, std::memory_order_relaxed);
-    return cudaGetLastError();
+    return el;
 }
 
 template <int L, int MODE> static cudaError_t kc_field(const KCParams<double>& p, cudaStream_t st) {

@@ -179,6 +179,8 @@ __global__ void __launch_bounds__(KCSGeom<L>::THREADS, 1)
     C* dt = reinterpret_cast<C*>(smem_staged + SG::DT_OFF);
     XA::dt_init(dt, (int)threadIdx.x, SG::THREADS);
     __syncthreads();
+    if constexpr (INV) pdl_go();  // the row pass takes each SM as it falls free; a scan (after the forward pass) waits
+    pdl_wait();
     // the first tile is copied by group 1 (whose own first tile comes later)
     if (grp == 1 && (int)blockIdx.x < ntiles) kcs_fetch<L, PRE>(p, blockIdx.x, stage, &nslot[0], &bar[0], tid);
 

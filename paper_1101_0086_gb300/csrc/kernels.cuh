@@ -207,6 +207,9 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
     const int N1m = p.N1 - 1;
     constexpr bool FAST = sizeof(T) == 4;  // FP32: finite-difference phases + polynomial exp
 
+    // passes that a scan follows let it start only at their end (pdl_go)
+    constexpr bool EARLY = F > 0 || MODE == KC_MPA_PRE || MODE == KC_INV;
+    if constexpr (EARLY) pdl_go();
     tw_init<T, L>(thi, tlo, tid, NT);
     if constexpr (INV) {
         // W_N^{-n2 k1} for the tile's columns: olo[m][g] = W^{-k1 m}, ohi[h][g] = W^{-k1 32 h}
@@ -218,6 +221,7 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
         }
     }
     __syncthreads();
+    pdl_wait();
 
     // ---- load: element j + r L/R0 of column col0 + g, straight into registers
     C vin[XA::Q0][XA::R0];
@@ -312,6 +316,7 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
         XI::run(vin, vout, s, thi, tlo);
     }
 
+    if constexpr (!EARLY) pdl_go();
     // ---- epilogue and store: element j + r L/RO of column col0 + g
 #pragma unroll
     for (int q = 0; q < QO; ++q) {
@@ -382,6 +387,7 @@ __global__ void __launch_bounds__(KRGeom<T, L, F>::NT, KRGeom<T, L, F>::NT <= 25
     const int tid = threadIdx.x;
     const long long row0 = (long long)blockIdx.x * G;
 
+    pdl_go();
     tw_init<T, L>(thi, tlo, tid, NT);
     if constexpr (FWD) {
         // W_N^{+n2 k1} for the tile's rows: olo[g][m] = W^{n2 m}, ohi[g][h] = W^{n2 128 h}
@@ -393,6 +399,7 @@ __global__ void __launch_bounds__(KRGeom<T, L, F>::NT, KRGeom<T, L, F>::NT <= 25
         }
     }
     __syncthreads();
+    pdl_wait();
 
     C vin[XA::Q0][XA::R0];
 #pragma unroll
@@ -515,8 +522,7 @@ template <typename T, int L> struct KNGeom {
     typedef KRGeom<T, L> R;
     static constexpr int G = R::G, TE = R::TE, NT = R::NT;
     typedef Tiling<T, 1> P;
-    static constexpr size_t smem_bytes =
-        ((size_t)TE + (TE >> P::PSH) + 1 + Tw<T, L>::N) * sizeof(cx<T>);
+    static constexpr size_t smem_bytes = ((size_t)TE + (TE >> P::PSH) + 1 + Tw<T, L>::N) * sizeof(cx<T>);
 };
 
 // The node rows row0 .. row0 + G - 1 of a launch (one tile) through steps
@@ -538,6 +544,7 @@ __device__ __forceinline__ void kn_tile(const KNParams<T>& p, long long row0, un
 
     tw_init<T, L>(thi, tlo, tid, NT);
     __syncthreads();
+    if constexpr (!CG) pdl_wait();  // CG: called inside the persistent kernel
 
     // ---- load node spectra (natural order, k = element index) and step 2
     C vin[XI::Q0][XI::R0];
@@ -588,6 +595,7 @@ __device__ __forceinline__ void kn_tile(const KNParams<T>& p, long long row0, un
     C vout[XF::QL][XF::RL];
     XF::run(vm, vout, s, thi, tlo);
 
+    if constexpr (!CG) pdl_go();
     // ---- V_j (Eq. (6)) and the store, natural order
 #pragma unroll
     for (int q = 0; q < XF::QL; ++q) {
@@ -1182,10 +1190,12 @@ __device__ __forceinline__ void scan_freq(const ScanParams<T>& p, int l, long lo
     // D = R_M - V_M/2 at node M in FP64 (psi_M = psi_0 + i D)
     const double sx = ((double)r.x - (double)c.x) - 0.5 * (double)vl.x;
     const double sy = ((double)r.y - (double)c.y) - 0.5 * (double)vl.y;
+    if constexpr (!CG) pdl_go();
     scan_node_m<T, CG, true>(p, l, i, k, p0, sx, sy, nblk);
 }
 
 template <typename T, bool PH> __global__ void __launch_bounds__(256) scan_kernel(const ScanParams<T> p) {
+    pdl_wait();
     scan_freq<T, false, PH>(p, blockIdx.y, (long long)blockIdx.x * blockDim.x + threadIdx.x, gridDim.x);
 }
 
@@ -1238,6 +1248,7 @@ constexpr int SCAN_S = 16, SCAN_NT = 128;
 template <bool STORE> __global__ void __launch_bounds__(SCAN_NT, 5) scan_pair_kernel(const ScanParams<float> p) {
     __shared__ float4 ring[SCAN_S * SCAN_NT];
     __shared__ float4 cst[SCAN_NT];  // PairWalk::consts of the nodes at hand
+    pdl_wait();
     const int l = blockIdx.y;
     const long long i = 2 * ((long long)blockIdx.x * SCAN_NT + threadIdx.x);
     const long long lo = (long long)l * p.N, N2 = p.N >> 1;  // N2: float4 distance of nodes
@@ -1311,6 +1322,7 @@ template <bool STORE> __global__ void __launch_bounds__(SCAN_NT, 5) scan_pair_ke
         }
     }
     cp_async_wait_group<0>();
+    pdl_go();
     // D = R_M - V_M/2 at node M in FP64 (psi_M = psi_0 + i D)
     scan_pair_m<true>(p, l, i, k, pa, pb, ((double)ra.x - (double)ca.x) - 0.5 * (double)va.x,
                       ((double)ra.y - (double)ca.y) - 0.5 * (double)va.y, ((double)rb.x - (double)cb.x) - 0.5 * (double)vb.x,
@@ -1335,6 +1347,7 @@ __global__ void __launch_bounds__(32 * SCS_W, sizeof(T) == 4 ? 4 : 2) scan_split
     constexpr bool F32 = sizeof(T) == 4;
     constexpr int SCS_C = F32 ? 16 : 8;         // nodes a thread holds
     __shared__ C ps[SCS_W][32], pc[SCS_W][32];  // the runs' sums and compensations
+    pdl_wait();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, l = blockIdx.y;
     const long long i = (long long)blockIdx.x * 32 + lane;
     const long long lo = (long long)l * p.N;
@@ -1371,6 +1384,7 @@ __global__ void __launch_bounds__(32 * SCS_W, sizeof(T) == 4 ? 4 : 2) scan_split
             }
         }
         if (jb > 1) __syncthreads();  // the previous panel's sums have been read
+        if (jb + SCS_W * run > p.M) pdl_go();
         ps[w][lane] = s;
         if constexpr (F32) pc[w][lane] = sc;
         __syncthreads();
@@ -1417,6 +1431,8 @@ template <typename T>
 __global__ void __launch_bounds__(256) transpose_kernel(const cx<T>* __restrict__ in, cx<T>* __restrict__ out,
                                                          long long R, long long Cc) {
     __shared__ cx<T> t[32][33];
+    pdl_go();
+    pdl_wait();
     const long long r0 = (long long)blockIdx.y * 32, c0 = (long long)blockIdx.x * 32;
     for (int y = threadIdx.y; y < 32; y += 8) {
         const long long r = r0 + y, c = c0 + threadIdx.x;
@@ -1432,6 +1448,8 @@ __global__ void __launch_bounds__(256) transpose_kernel(const cx<T>* __restrict_
 // Precision conversions between the FP64 state and working buffers.
 template <typename T>
 __global__ void __launch_bounds__(256) to_state_kernel(const cx<T>* in, double2* state, cx<T>* copy, long long N) {
+    pdl_go();
+    pdl_wait();
     const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= N) return;
     const cx<T> v = in[k];
@@ -1440,6 +1458,8 @@ __global__ void __launch_bounds__(256) to_state_kernel(const cx<T>* in, double2*
 }
 template <typename T>
 __global__ void __launch_bounds__(256) from_state_kernel(const double2* state, cx<T>* out, long long N) {
+    pdl_go();
+    pdl_wait();
     const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= N) return;
     const double2 v = state[k];

@@ -19,7 +19,7 @@ static cudaError_t kn_one(const KNParams<float>& p, cudaStream_t st) {
     if (nblk <= 0) return cudaSuccess;
     const bool prof = g_prof_on.load(std::memory_order_relaxed);
     if (prof) prof_begin(st);
-    kn_kernel<float, L, PIN, POUT><<<(unsigned)nblk, Gm::NT, Gm::smem_bytes, st>>>(p);
+    const cudaError_t el = launch_pdl(pdl_fills(nblk), kn_kernel<float, L, PIN, POUT>, (unsigned)nblk, Gm::NT, Gm::smem_bytes, st, p);
     if (prof) {
         // every node read once and written once (a shared psi_0 once per link)
         const double cs = (double)sizeof(cx<float>), nodes = (double)p.nrows;
@@ -27,7 +27,7 @@ static cudaError_t kn_one(const KNParams<float>& p, cudaStream_t st) {
         prof_end(PK_KN, st, (rd + nodes) * L * cs);
     }
     g_launches.fetch_add(1, std::memory_order_relaxed);
-    return cudaGetLastError();
+    return el;
 }
 
 template <int L> static cudaError_t kn_len(const KNParams<float>& p, cudaStream_t st) {

@@ -31,10 +31,10 @@ static cudaError_t krs_one(const KRParams<float>& p, cudaStream_t st) {
     const unsigned grid = (unsigned)(ntiles < sms ? ntiles : sms);  // one CTA per SM
     const bool prof = g_prof_on.load(std::memory_order_relaxed);
     if (prof) prof_begin(st);
-    krs_kernel<L, MODE><<<grid, SG::THREADS, SG::smem_bytes, st>>>(p, p.spin_limit);
+    const cudaError_t el = launch_pdl(true, krs_kernel<L, MODE>, grid, SG::THREADS, SG::smem_bytes, st, p, p.spin_limit);
     if (prof) prof_end(prof_kr_kind(MODE), st, 2.0 * (double)p.nrows * L * sizeof(cx<float>));
     g_launches.fetch_add(1, std::memory_order_relaxed);
-    return cudaGetLastError();
+    return el;
 }
 
 template <int L>
@@ -64,10 +64,10 @@ static cudaError_t kr_one(const KRParams<float>& p, cudaStream_t st) {
     if (nblk <= 0) return cudaSuccess;
     const bool prof = g_prof_on.load(std::memory_order_relaxed);
     if (prof) prof_begin(st);
-    kr_kernel<float, L, MODE, F><<<(unsigned)nblk, Gm::NT, Gm::smem_bytes, st>>>(p);
+    const cudaError_t el = launch_pdl(true, kr_kernel<float, L, MODE, F>, (unsigned)nblk, Gm::NT, Gm::smem_bytes, st, p);
     if (prof) prof_end(prof_kr_kind(MODE), st, 2.0 * (double)p.nrows * L * sizeof(cx<float>));
     g_launches.fetch_add(1, std::memory_order_relaxed);
-    return cudaGetLastError();
+    return el;
 }
 
 template <int L, int MODE> static cudaError_t kr_field(const KRParams<float>& p, cudaStream_t st) {

@@ -21,10 +21,10 @@ static cudaError_t kr_one(const KRParams<double>& p, cudaStream_t st) {
     if (nblk <= 0) return cudaSuccess;
     const bool prof = g_prof_on.load(std::memory_order_relaxed);
     if (prof) prof_begin(st);
-    kr_kernel<double, L, MODE, F><<<(unsigned)nblk, Gm::NT, Gm::smem_bytes, st>>>(p);
+    const cudaError_t el = launch_pdl(F == 0 || pdl_field<double>(p.N), kr_kernel<double, L, MODE, F>, (unsigned)nblk, Gm::NT, Gm::smem_bytes, st, p);
     if (prof) prof_end(prof_kr_kind(MODE), st, 2.0 * (double)p.nrows * L * sizeof(cx<double>));
     g_launches.fetch_add(1, std::memory_order_relaxed);
-    return cudaGetLastError();
+    return el;
 }
 
 template <int L, int MODE> static cudaError_t kr_field(const KRParams<double>& p, cudaStream_t st) {

@@ -157,6 +157,8 @@ __global__ void __launch_bounds__(KRSGeom<L>::THREADS, 1) krs_kernel(const KRPar
     }
     tw_init<float, L>(thi, tlo, (int)threadIdx.x, SG::THREADS);
     __syncthreads();
+    pdl_go();
+    pdl_wait();
     int last_copy = -1;  // CTA-local index of the last tile this thread started copying
     if (threadIdx.x == 0 && (int)blockIdx.x < ntiles) {
         krs_fetch<L>(p, blockIdx.x, stage, &bar[0]);

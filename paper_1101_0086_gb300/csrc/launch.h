@@ -44,6 +44,38 @@ template <class F> inline cudaError_t attrs_once(AttrOnce& once, F&& set) {
     return e;
 }
 
+// Launch of a kernel that calls pdl_wait() before its first global access
+// (device.cuh): its launch and preparation overlap the end of the kernel
+// before it in the stream.  Split step of 2^14 modes (two kernels whose tables
+// and launches took longer than their transforms) 13.9 -> 6.2 us, one span of
+// a 2^16 link 3.94 -> 3.66 ms.  early = false: an ordinary launch.
+template <class... P, class... A>
+inline cudaError_t launch_pdl(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                              A... args) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cudaLaunchAttribute a{};
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &a;
+    c.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+// Whether a level's kernel of `blocks` blocks starts early: a grid that does
+// not fill the SMs twice over would be packed onto the first ones that fall
+// free (one span of a 2^12 link, 72 blocks of node transforms and 128 of the
+// scan: 761 us with ordinary launches, 861 to 940 with early ones).
+inline bool pdl_fills(long long blocks) { return blocks >= 2 * 152; }
+// Whether a pass over a single field of n samples starts early.  FP64 passes of
+// 2^16 .. 2^18 samples, bound by the schedulers they spread over, would be
+// packed too: us a split step, early / ordinary: 2^14 27 / 46, 2^15 31 / 43,
+// 2^16 86 / 42, 2^17 157 / 68, 2^18 189 / 123, 2^20 412 / 419; FP32: 2^14 6.2 /
+// 13.9, 2^18 12.9 / 13.8, 2^20 23.3 / 23.2, 2^22 66 / 71.
+template <typename T> inline bool pdl_field(long long n) { return sizeof(T) == 4 || n <= (1ll << 15) || n > (1ll << 18); }
+
 // Optional CUDA-event timing of every launch, by kernel kind (off by
 // default; enabled through mpa_profile).
 enum {

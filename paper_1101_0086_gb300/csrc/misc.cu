@@ -194,14 +194,14 @@ template <typename T> cudaError_t scan_launch(const ScanParams<T>& p, int p_link
     const bool pr = g_prof_on.load(std::memory_order_relaxed);
     if (pr) prof_begin(st);
     const dim3 grid(blocks_for(p.N, 256), (unsigned)p_links), split(blocks_for(p.N, 32), (unsigned)p_links);
-    if constexpr (sizeof(T) == 4) {
-        if (!p.phases) scan_split_kernel<T><<<split, 32 * SCS_W, 0, st>>>(p);
-        else if (p.mode == 0) scan_pair_kernel<true><<<grid, SCAN_NT, 0, st>>>(p);
-        else scan_pair_kernel<false><<<grid, SCAN_NT, 0, st>>>(p);
+    const bool early = pdl_fills((long long)grid.x * grid.y);
+    cudaError_t el;
+    if (!p.phases && (sizeof(T) == 4 || p.N * p_links <= kScanSplit64Max)) {
+        el = launch_pdl(pdl_fills((long long)split.x * split.y), scan_split_kernel<T>, split, 32 * SCS_W, 0, st, p);
+    } else if constexpr (sizeof(T) == 4) {
+        el = launch_pdl(early, p.mode == 0 ? scan_pair_kernel<true> : scan_pair_kernel<false>, grid, SCAN_NT, 0, st, p);
     } else {
-        if (p.phases) scan_kernel<T, true><<<grid, 256, 0, st>>>(p);
-        else if (p.N * p_links <= kScanSplit64Max) scan_split_kernel<T><<<split, 32 * SCS_W, 0, st>>>(p);
-        else scan_kernel<T, false><<<grid, 256, 0, st>>>(p);
+        el = launch_pdl(early, p.phases ? scan_kernel<T, true> : scan_kernel<T, false>, grid, 256, 0, st, p);
     }
     if (pr) {
         const double cs = (double)sizeof(cx<T>), n = (double)p.N;
@@ -212,31 +212,31 @@ template <typename T> cudaError_t scan_launch(const ScanParams<T>& p, int p_link
         prof_end(PK_SCAN, st, b);
     }
     g_launches.fetch_add(1, std::memory_order_relaxed);
-    return cudaGetLastError();
+    return el;
 }
 
 template <typename T>
 cudaError_t transpose_launch(const cx<T>* in, cx<T>* out, long long R, long long C, cudaStream_t st) {
     if (const cudaError_t eg = launch_gate()) return eg;
     dim3 grid((unsigned)((C + 31) / 32), (unsigned)((R + 31) / 32));
-    transpose_kernel<T><<<grid, dim3(32, 8), 0, st>>>(in, out, R, C);
+    const cudaError_t el = launch_pdl(true, transpose_kernel<T>, grid, dim3(32, 8), 0, st, in, out, R, C);
     g_launches.fetch_add(1, std::memory_order_relaxed);
-    return cudaGetLastError();
+    return el;
 }
 
 template <typename T>
 cudaError_t to_state_launch(const cx<T>* in, double2* state, cx<T>* copy, long long N, cudaStream_t st) {
     if (const cudaError_t eg = launch_gate()) return eg;
-    to_state_kernel<T><<<blocks_for(N, 256), 256, 0, st>>>(in, state, copy, N);
+    const cudaError_t el = launch_pdl(true, to_state_kernel<T>, blocks_for(N, 256), 256, 0, st, in, state, copy, N);
     g_launches.fetch_add(1, std::memory_order_relaxed);
-    return cudaGetLastError();
+    return el;
 }
 
 template <typename T> cudaError_t from_state_launch(const double2* state, cx<T>* out, long long N, cudaStream_t st) {
     if (const cudaError_t eg = launch_gate()) return eg;
-    from_state_kernel<T><<<blocks_for(N, 256), 256, 0, st>>>(state, out, N);
+    const cudaError_t el = launch_pdl(true, from_state_kernel<T>, blocks_for(N, 256), 256, 0, st, state, out, N);
     g_launches.fetch_add(1, std::memory_order_relaxed);
-    return cudaGetLastError();
+    return el;
 }
 
 template cudaError_t scan_launch<float>(const ScanParams<float>&, int, cudaStream_t);

@@ -86,3 +86,34 @@ def test_fp32_split_step(M, logn):
     M.ss_propagate(d, dm_map(1), T, 0.05, 44.8, 45.2)
     ref = oracle.ss(a.astype(np.complex128), dm_map(1), T, 44.8, 45.2, 0.05)
     assert oracle.rel_l2(d.cpu().numpy(), ref) < 2e-5
+
+
+@pytest.mark.parametrize("what", ["ss", "link14", "link18"])
+def test_captured_passes_replay(M, what):
+    """Kernels that start early (launch_pdl) under stream capture: a replay
+    gives the direct call's result, bit for bit."""
+    import torch
+    logn = {"ss": 13, "link14": 14, "link18": 18}[what]
+    n = 1 << logn
+    T = 100.0 * n / 128
+    a = torch.from_numpy(wdm_field(n, T, 4, 50.0, n // 128, 30.0, 2.0, "qpsk", seed=1)).to(torch.complex64).cuda()
+    ws = torch.empty(M.ss_workspace_bytes(n, "fp32"), dtype=torch.uint8, device="cuda")
+    plan = M.Plan(dm_map(1), n, T, 5.0, 12, 2)
+
+    def run(x):
+        if what == "ss":
+            M.ss_propagate(x, dm_map(1), T, 0.05, 44.8, 45.2, workspace=ws)
+        else:
+            plan.propagate(x, 40.0, 50.0)
+
+    want = a.clone()
+    run(want)
+    x = a.clone()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        run(x)
+    for _ in range(2):
+        x.copy_(a)
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(torch.view_as_real(x), torch.view_as_real(want))
