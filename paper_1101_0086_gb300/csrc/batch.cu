@@ -153,10 +153,11 @@ int run_group(mpa_batch* b, Group& g, cudaStream_t st) {
     // a fresh increment check per propagation (a run that ended early, e.g.
     // on a timeout, must not leave a half-counted level behind)
     MPA_TRY(cudaMemsetAsync(mon.conv, 0, (size_t)n * sizeof(ConvState), st));
-    // A_hat(0) = F[A] for every link (its node-0 buffer is the scratch)
+    // A_hat(0) = F[A] for every link (its first two node buffers are the scratch)
     for (int i = 0; i < n; ++i) {
         cx<T>* scratch = psi + (long long)i * (M + 1) * N;
-        int rc = fft_forward<T>(s, reinterpret_cast<const cx<T>*>(b->links[(size_t)g.links[(size_t)i]].field), scratch, st);
+        int rc = fft_forward<T>(N, reinterpret_cast<const cx<T>*>(b->links[(size_t)g.links[(size_t)i]].field), scratch,
+                                scratch + N, st);
         if (rc) return rc;
         MPA_TRY(to_state_launch<T>(scratch, state + (long long)i * N, sizeof(T) == 4 ? psi0c + (long long)i * N : nullptr,
                                    N, st));
@@ -176,7 +177,7 @@ int run_group(mpa_batch* b, Group& g, cudaStream_t st) {
     for (int i = 0; i < n; ++i) {
         cx<T>* scratch = psi + (long long)i * (M + 1) * N;
         MPA_TRY(from_state_launch<T>(state + (long long)i * N, scratch, N, st));
-        int rc = fft_inverse<T>(s, scratch, reinterpret_cast<cx<T>*>(b->links[(size_t)g.links[(size_t)i]].field), st);
+        int rc = fft_inverse<T>(N, scratch, reinterpret_cast<cx<T>*>(b->links[(size_t)g.links[(size_t)i]].field), scratch, st);
         if (rc) return rc;
     }
     return MPA_OK;

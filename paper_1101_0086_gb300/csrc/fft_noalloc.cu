@@ -74,13 +74,11 @@ extern "C" int mpa_fft_noalloc(int64_t N, int32_t precision, int32_t sign, void*
     if (precision == MPA_FP32) {
         float2* d = reinterpret_cast<float2*>(data);
         float2* w = reinterpret_cast<float2*>(scratch);
-        rc = sign > 0 ? fft_forward<float>(s, d, w, st) : fft_inverse<float>(s, d, w, st);
+        rc = sign > 0 ? fft_forward<float>(N, d, d, w, st) : fft_inverse<float>(N, d, d, w, st);
     } else {
         double2* d = reinterpret_cast<double2*>(data);
         double2* w = reinterpret_cast<double2*>(scratch);
-        rc = sign > 0 ? fft_forward<double>(s, d, w, st) : fft_inverse<double>(s, d, w, st);
+        rc = sign > 0 ? fft_forward<double>(N, d, d, w, st) : fft_inverse<double>(N, d, d, w, st);
     }
-    if (rc) return rc;
-    MPA_TRY(cudaMemcpyAsync(data, scratch, bytes, cudaMemcpyDeviceToDevice, st));
-    return MPA_OK;
+    return rc;
 }

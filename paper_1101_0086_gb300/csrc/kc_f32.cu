@@ -49,7 +49,7 @@ template <int L> static bool kcs_fits(const KCParams<float>& p) {
 }
 
 bool kc_staged(int mode, int logL, const KCParams<float>& p) {
-    if (!MPA_KC_STAGED || !p.err || mode == KC_SS_STEP || mode == KC_MPA_POST || p.npl <= 0) return false;
+    if (!MPA_KC_STAGED || !p.err || (mode != KC_MPA_PRE && mode != KC_INV && mode != KC_FWD) || p.npl <= 0) return false;
     switch (logL) {
         case 8: return kcs_fits<256>(p);
         case 9: return kcs_fits<512>(p);
@@ -124,6 +124,9 @@ static cudaError_t kc_mode(int mode, const KCParams<float>& p, cudaStream_t st) 
         case KC_SS_STEP: return kc_field<L, KC_SS_STEP>(p, st);
         case KC_FWD: return p.err ? kc_one<L, KC_FWD>(p, st) : kc_field<L, KC_FWD>(p, st);
         case KC_INV: return p.err ? kc_one<L, KC_INV>(p, st) : kc_field<L, KC_INV>(p, st);
+        case KC_FWDF: return kc_field<L, KC_FWDF>(p, st);
+        case KC_FWD_T: return kc_field<L, KC_FWD_T>(p, st);
+        case KC_INV_T: return kc_field<L, KC_INV_T>(p, st);
     }
     return cudaErrorInvalidValue;
 }

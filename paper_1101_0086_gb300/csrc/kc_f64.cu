@@ -49,6 +49,9 @@ static cudaError_t kc_mode(int mode, const KCParams<double>& p, cudaStream_t st)
         case KC_SS_STEP: return kc_field<L, KC_SS_STEP>(p, st);
         case KC_FWD: return p.err ? kc_one<L, KC_FWD>(p, st) : kc_field<L, KC_FWD>(p, st);
         case KC_INV: return p.err ? kc_one<L, KC_INV>(p, st) : kc_field<L, KC_INV>(p, st);
+        case KC_FWDF: return kc_field<L, KC_FWDF>(p, st);
+        case KC_FWD_T: return kc_field<L, KC_FWD_T>(p, st);
+        case KC_INV_T: return kc_field<L, KC_INV_T>(p, st);
     }
     return cudaErrorInvalidValue;
 }

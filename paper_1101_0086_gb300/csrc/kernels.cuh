@@ -15,6 +15,9 @@
 //                             MPA_POST forward -> exp(-i beta_j) * sigma dz / exp(int G)  (V_j of Eq. (6))
 //                             SS_STEP  forward -> linear step of Eq. (4) -> inverse
 //                             FWD      forward only        INV  inverse only
+//                             FWDF     forward, then the outer factor W_N^{+n2 k1}
+//                             FWD_T, INV_T  the second pass of a transform between natural orders:
+//                                      column c is the source's contiguous row c
 //   KR (row pass)     modes: MPA  inverse -> 1/N -> |A|^2 A -> forward
 //                             SS   inverse -> 1/N -> A exp(i s |A|^2) -> forward
 //                             FWD  forward only        INV  inverse -> 1/N
@@ -29,7 +32,7 @@
 
 namespace mpa {
 
-enum { KC_MPA_PRE = 0, KC_MPA_POST = 1, KC_SS_STEP = 2, KC_FWD = 3, KC_INV = 4 };
+enum { KC_MPA_PRE = 0, KC_MPA_POST = 1, KC_SS_STEP = 2, KC_FWD = 3, KC_INV = 4, KC_FWDF = 5, KC_FWD_T = 6, KC_INV_T = 7 };
 // KR_MPA_KEEP: KR_MPA that also writes A(t) to keep (the reverse mode's
 // forward recompute keeps it for the adjoint of the Kerr term)
 enum { KR_MPA = 0, KR_SS = 1, KR_FWD = 2, KR_INV = 3, KR_MPA_KEEP = 4 };
@@ -135,6 +138,12 @@ template <typename T, int L, int F = 0> struct KRGeom {
     static constexpr size_t smem_bytes = smem_elems * sizeof(cx<T>);
 };
 
+// 2^-n
+template <typename T> __device__ __forceinline__ T pow2_neg(int n) {
+    if constexpr (sizeof(T) == 4) return __int_as_float((127 - n) << 23);
+    else return __longlong_as_double((long long)(1023 - n) << 52);
+}
+
 __device__ __forceinline__ long long signed_k(long long k, long long N) { return k < (N >> 1) ? k : k - N; }
 
 // Global load of data another CTA of the same (persistent) kernel may have
@@ -188,8 +197,10 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
     typedef KCGeom<T, L, F> Gm;
     typedef typename Gm::P P;
     constexpr int G = Gm::G, TE = Gm::TE, NT = Gm::NT;
-    constexpr bool FWD = (MODE == KC_MPA_POST || MODE == KC_SS_STEP || MODE == KC_FWD);
-    constexpr bool INV = (MODE == KC_MPA_PRE || MODE == KC_SS_STEP || MODE == KC_INV);
+    constexpr bool FWD = (MODE == KC_MPA_POST || MODE == KC_SS_STEP || MODE == KC_FWD || MODE == KC_FWDF || MODE == KC_FWD_T);
+    constexpr bool INV = (MODE == KC_MPA_PRE || MODE == KC_SS_STEP || MODE == KC_INV || MODE == KC_INV_T);
+    constexpr bool ROWS = (MODE == KC_FWD_T || MODE == KC_INV_T);  // columns are the source's rows
+    constexpr bool FAC = (INV || MODE == KC_FWDF) && !ROWS;        // outer factor at the store
     // forward: small radix first, so it ends with an RMAX pass that meets the
     // inverse's first RMAX pass in registers (split-step column pass)
     typedef Xform<T, L, G, NT, P::RMAX, +1, LAYOUT_COL, P::PSH, true> XF;
@@ -211,11 +222,11 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
     constexpr bool EARLY = F > 0 || MODE == KC_MPA_PRE || MODE == KC_INV;
     if constexpr (EARLY) pdl_go();
     tw_init<T, L>(thi, tlo, tid, NT);
-    if constexpr (INV) {
-        // W_N^{-n2 k1} for the tile's columns: olo[m][g] = W^{-k1 m}, ohi[h][g] = W^{-k1 32 h}
+    if constexpr (FAC) {
+        // W_N^{-n2 k1} for the tile's columns: olo[m][g] = W^{-k1 m}, ohi[h][g] = W^{-k1 32 h} (FWDF: +)
         for (int i = tid; i < G * (Gm::OLO + Gm::OHI); i += NT) {
             const int g = i % G, m = i / G;
-            const long long k1 = (col0 + g) & N1m;
+            const long long k1 = MODE == KC_FWDF ? -((col0 + g) & N1m) : (col0 + g) & N1m;
             if (m < Gm::OLO) olo[m * G + g] = expi_ratio<T>(-k1 * m, p.logN);
             else ohi[(m - Gm::OLO) * G + g] = expi_ratio<T>(-k1 * ((long long)(m - Gm::OLO) << Gm::OSH), p.logN);
         }
@@ -234,8 +245,10 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
         const int node = ok ? (int)(col >> p.logN1) : 0;
         const int l = node / p.npl, jn = node - l * p.npl;
         const long long c = col & N1m;
-        const C* src = (p.src0 && jn == 0) ? p.src0 + l * p.src0_lstride + c
-                                           : p.src + l * p.src_lstride + jn * p.src_stride + c;
+        const C* src = ROWS                  ? p.src + col * L
+                       : (p.src0 && jn == 0) ? p.src0 + l * p.src0_lstride + c
+                                             : p.src + l * p.src_lstride + jn * p.src_stride + c;
+        const long long rs = ROWS ? 1 : p.N1;  // distance of the column's rows
         NodeC nc{};
         if constexpr (MODE == KC_MPA_PRE) {
             if (MPA_DBG_OK(p.dbg, p.loff + l, sizeof(int)) && MPA_DBG_OK(p.dbg, p.nodes + p.loff[l] + jn, sizeof(NodeC)))
@@ -247,8 +260,7 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
 #pragma unroll
         for (int r = 0; r < XA::R0; ++r) {
             const int row = j + r * (L / XA::R0);
-            C v = ok && MPA_DBG_OK(p.dbg, src + (long long)row * p.N1, sizeof(C)) ? src[(long long)row * p.N1]
-                                                                                  : mkc(T(0), T(0));
+            C v = ok && MPA_DBG_OK(p.dbg, src + row * rs, sizeof(C)) ? src[row * rs] : mkc(T(0), T(0));
             if constexpr (MODE == KC_MPA_PRE) {
                 // MPA step 2: A_hat_j = psi_j exp(i beta(w, z_j) + int G)
                 C ph;
@@ -340,17 +352,18 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
         // multiple of the low table's length: one lookup per butterfly
         constexpr bool HOIST = (L / RO) % Gm::OLO == 0;
         C wlo = mkc(T(1), T(0));
-        if constexpr (INV && HOIST) wlo = olo[(j & (Gm::OLO - 1)) * G + g];
+        if constexpr (FAC && HOIST) wlo = olo[(j & (Gm::OLO - 1)) * G + g];
 #pragma unroll
         for (int r = 0; r < RO; ++r) {
             const int row = j + r * (L / RO);
             C v = vout[q][r];
-            if constexpr (INV) {
+            if constexpr (FAC) {
                 // four-step factor W_N^{-n2 k1}, n2 = row
                 C w = HOIST ? wlo : olo[(row & (Gm::OLO - 1)) * G + g];
                 if constexpr (Gm::OHI > 1) w = cmul(ohi[(row >> Gm::OSH) * G + g], w);
                 v = cmul(v, w);
             }
+            if constexpr (MODE == KC_INV_T) v = cscale(v, pow2_neg<T>(p.logN));
             if constexpr (MODE == KC_MPA_POST) {
                 // V_j = sigma(z_j) dz F[|A_j|^2 A_j] exp(-i beta(w, z_j) - int G)   (Eq. (6))
                 C ph;

@@ -360,7 +360,7 @@ int propagate_t(mpa_plan* p, void* field, double z_from, double z_to, cudaStream
     double2* state = reinterpret_cast<double2*>(p->ws + p->off_state);
     cx<T>* psi0c = reinterpret_cast<cx<T>*>(p->ws + p->off_psi0c);
     // A_hat(z_from) = F[A] -> FP64 state and its working copy
-    int rc = fft_forward<T>(s, f, psi, st);
+    int rc = fft_forward<T>(s.N, f, psi, psi + s.N, st);
     if (rc) return rc;
     MPA_TRY(to_state_launch<T>(psi, state, sizeof(T) == 4 ? psi0c : nullptr, s.N, st));
     for (long q = 0; q < n_int; ++q) {
@@ -372,7 +372,7 @@ int propagate_t(mpa_plan* p, void* field, double z_from, double z_to, cudaStream
     }
     // A(z_to) = F^-1[A_hat]
     MPA_TRY(from_state_launch<T>(state, psi, s.N, st));
-    return fft_inverse<T>(s, psi, f, st);
+    return fft_inverse<T>(s.N, psi, f, psi, st);
 }
 
 template <typename T>
@@ -790,19 +790,16 @@ int mpa_fft(int64_t N, int32_t precision, int32_t sign, void* data, void* worksp
     ss_workspace_size(N, precision, &need);
     if (ws_bytes < need) return MPA_ERR_WORKSPACE;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const size_t bytes = (size_t)N * (precision == MPA_FP32 ? sizeof(float2) : sizeof(double2));
     if (precision == MPA_FP32) {
         float2* d = reinterpret_cast<float2*>(data);
         float2* w = reinterpret_cast<float2*>(workspace);
-        rc = sign > 0 ? fft_forward<float>(s, d, w, st) : fft_inverse<float>(s, d, w, st);
+        rc = sign > 0 ? fft_forward<float>(N, d, d, w, st) : fft_inverse<float>(N, d, d, w, st);
     } else {
         double2* d = reinterpret_cast<double2*>(data);
         double2* w = reinterpret_cast<double2*>(workspace);
-        rc = sign > 0 ? fft_forward<double>(s, d, w, st) : fft_inverse<double>(s, d, w, st);
+        rc = sign > 0 ? fft_forward<double>(N, d, d, w, st) : fft_inverse<double>(N, d, d, w, st);
     }
-    if (rc) return rc;
-    MPA_TRY(cudaMemcpyAsync(data, workspace, bytes, cudaMemcpyDeviceToDevice, st));
-    return MPA_OK;
+    return rc;
 }
 
 double mpa_gamma_from_db_per_km(double db_per_km) { return db_per_km * std::log(10.0) / 20.0; }

@@ -549,9 +549,8 @@ def ss_propagate(field: torch.Tensor, fiber, T_ps: float, dz_km: float, z_from_k
     prec = _prec(field.dtype)
     N = field.numel()
     ptr = _field_ptr(field, _cdtype(prec), N, "ss_propagate")
-    need = ss_workspace_bytes(N, prec)
     if workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=field.device)
+        workspace = torch.empty(ss_workspace_bytes(N, prec), dtype=torch.uint8, device=field.device)
     wp = _ws_ptr(workspace, field.device, "ss_propagate")
     _on_device(field.device, "ss_propagate")
     fm, segs = _fiber_struct(fiber)
@@ -606,9 +605,8 @@ def fft(data: torch.Tensor, sign: int, workspace: Optional[torch.Tensor] = None,
     prec = _prec(data.dtype)
     N = data.numel()
     ptr = _field_ptr(data, _cdtype(prec), N, "fft")
-    need = ss_workspace_bytes(N, prec)
     if workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=data.device)
+        workspace = torch.empty(ss_workspace_bytes(N, prec), dtype=torch.uint8, device=data.device)
     wp = _ws_ptr(workspace, data.device, "fft")
     _on_device(data.device, "fft")
     _check(lib().mpa_fft(N, prec, int(sign), ptr, wp, workspace.numel(), _stream(stream)), "mpa_fft")

@@ -62,7 +62,7 @@ def test_fp64_interval(M, logn, split):
     assert oracle.rel_l2(d.cpu().numpy(), oracle.mpa(a, dm_map(1), T, 45.0, 50.0, 5.0, 6, 2)) < 1e-12
 
 
-@pytest.mark.parametrize("logn", [8, 10, 13, 16, 18, 19, 20, 22])
+@pytest.mark.parametrize("logn", [8, 10, 13, 16, 18, 19, 20, 22, 23])
 def test_fp32_transform_pair(M, logn):
     """Fine and medium tiles in FP32: 22 roundings at 6e-8 and their partial
     sums' growth, 4e-6."""
