@@ -896,6 +896,10 @@ template <> struct Tiling<double, 3> {
 template <> struct Tiling<double, 4> {
     static constexpr int E = 8, RMAX = 8, PSH = 3, CMIN = 1, TE = 256;
 };
+// KIND 5 = on-chip node transforms of few nodes (kn_fine).
+template <> struct Tiling<float, 5> {
+    static constexpr int E = 16, RMAX = 16, PSH = 4;
+};
 // The tiles of a single-field pass of length L over `elems` elements: 0 the
 // large tiles of the MPA passes, 1 fine, 2 medium.  Measured, us a split step
 // (both passes), large / medium / fine.  FP32 (launches and latency, then

@@ -531,20 +531,22 @@ template <typename T> struct KNParams {
     DbgRange dbg;  // checked range of the debug build
 };
 
-template <typename T, int L> struct KNGeom {
+// F = 1 (FP32): one node a CTA (several below 2^10 modes), 16 elements a
+// thread, for launches whose large tiles would not fill the SMs twice (kn_fine).
+template <typename T, int L, int F = 0> struct KNGeom {
     typedef KRGeom<T, L> R;
-    static constexpr int G = R::G, TE = R::TE, NT = R::NT;
-    typedef Tiling<T, 1> P;
+    typedef Tiling<T, F ? 5 : 1> P;
+    static constexpr int G = F ? (L >= 1024 ? 1 : 1024 / L) : R::G, TE = G * L, NT = TE / P::E;
     static constexpr size_t smem_bytes = ((size_t)TE + (TE >> P::PSH) + 1 + Tw<T, L>::N) * sizeof(cx<T>);
 };
 
 // The node rows row0 .. row0 + G - 1 of a launch (one tile) through steps
 // 2-4 and the weight of Eq. (6); the block's threads and shared memory.
-template <typename T, int L, bool CG, bool PIN, bool POUT>
+template <typename T, int L, bool CG, bool PIN, bool POUT, int F = 0>
 __device__ __forceinline__ void kn_tile(const KNParams<T>& p, long long row0, unsigned char* smem_raw) {
     typedef cx<T> C;
-    typedef KNGeom<T, L> Gm;
-    typedef Tiling<T, 1> P;
+    typedef KNGeom<T, L, F> Gm;
+    typedef typename Gm::P P;
     constexpr int G = Gm::G, NT = Gm::NT, TE = Gm::TE;
     typedef Xform<T, L, G, NT, P::RMAX, -1, LAYOUT_ROW, P::PSH, false> XI;
     typedef Xform<T, L, G, NT, P::RMAX, +1, LAYOUT_ROW, P::PSH, true> XF;
@@ -643,11 +645,11 @@ __device__ __forceinline__ void kn_tile(const KNParams<T>& p, long long row0, un
     }
 }
 
-template <typename T, int L, bool PIN, bool POUT>
-__global__ void __launch_bounds__(KNGeom<T, L>::NT, KNGeom<T, L>::NT <= 256 ? MPA_KR_MINB : 1)
+template <typename T, int L, bool PIN, bool POUT, int F = 0>
+__global__ void __launch_bounds__(KNGeom<T, L, F>::NT, KNGeom<T, L, F>::NT <= 256 ? MPA_KR_MINB : 1)
     kn_kernel(const KNParams<T> p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    kn_tile<T, L, false, PIN, POUT>(p, (long long)blockIdx.x * KNGeom<T, L>::G, smem_raw);
+    kn_tile<T, L, false, PIN, POUT, F>(p, (long long)blockIdx.x * KNGeom<T, L, F>::G, smem_raw);
 }
 
 // ------------------------------------------------------------------

@@ -119,3 +119,10 @@ def test_scan_with_phases_of_links_with_different_maps(M):
     assert b.status_code() == 0
     for x, r in zip(bufs, refs):
         assert oracle.rel_l2(x.cpu().numpy().astype(np.complex128), r) < TOL["fp32"]
+
+
+@pytest.mark.parametrize("logn,nodes", [(8, 3), (9, 1), (10, 142), (11, 7), (11, 1300), (12, 5), (12, 620)])
+def test_onchip_tiles_of_few_and_many_nodes(M, logn, nodes):
+    """On-chip node transforms on their fine tiles (fewer than 304 large tiles
+    of nodes) and on the large ones, the last tile partly filled."""
+    _propagate_against_oracle(M, 1 << logn, "fp32", dm_map(1), nodes, 2, 0)
