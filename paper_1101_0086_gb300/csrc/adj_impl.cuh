@@ -10,7 +10,7 @@ namespace adj {
 template <typename T, int L, int MODE>
 cudaError_t kca_one(const KCAParams<T>& p, cudaStream_t st) {
     if (const cudaError_t eg = launch_gate()) return eg;
-    typedef KCGeom<T, L> Gm;
+    typedef KCGeom<T, L, kca_tiles<T>(L)> Gm;
     static AttrOnce once;
     const cudaError_t ea = attrs_once(once, [] {
         cudaError_t e = cudaFuncSetAttribute(kca_kernel<T, L, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -281,14 +281,14 @@ cudaError_t kra_any(int logL, const KRAParams<T>& p, cudaStream_t st) {
 template <typename T>
 int kca_cols(int logL) {
     switch (logL) {
-        case 4: return KCGeom<T, 16>::G;
-        case 5: return KCGeom<T, 32>::G;
-        case 6: return KCGeom<T, 64>::G;
-        case 7: return KCGeom<T, 128>::G;
-        case 8: return KCGeom<T, 256>::G;
-        case 9: return KCGeom<T, 512>::G;
-        case 10: return KCGeom<T, 1024>::G;
-        case 11: return KCGeom<T, 2048>::G;
+        case 4: return KCGeom<T, 16, kca_tiles<T>(16)>::G;
+        case 5: return KCGeom<T, 32, kca_tiles<T>(32)>::G;
+        case 6: return KCGeom<T, 64, kca_tiles<T>(64)>::G;
+        case 7: return KCGeom<T, 128, kca_tiles<T>(128)>::G;
+        case 8: return KCGeom<T, 256, kca_tiles<T>(256)>::G;
+        case 9: return KCGeom<T, 512, kca_tiles<T>(512)>::G;
+        case 10: return KCGeom<T, 1024, kca_tiles<T>(1024)>::G;
+        case 11: return KCGeom<T, 2048, kca_tiles<T>(2048)>::G;
     }
     return -1;
 }

@@ -35,6 +35,19 @@ struct AdjLayout {
 
 int n_periods_of(const HostMap& m) { return (int)std::lround(m.length / m.period); }
 
+// The split of the recompute and reverse passes (the forward pass keeps the
+// plan's): FP32 columns of 2^8 points, rows up to 2^12.  The reverse column
+// passes hold two fields and are bound by registers: 256 points 770 us a
+// launch of 2^20 x 143 nodes, 512 862 us, 1024 1100 us, which outweighs the
+// longer rows (a gradient over 10 km of the 2^20 link 26.8, 28.3, 29.1 ms with
+// everything at that split).
+Split reverse_split(const mpa_plan* p) {
+    Split s;
+    const int l = p->sp.logN - 12 > 8 ? p->sp.logN - 12 : 8;
+    if (p->prec != MPA_FP32 || l >= p->sp.logN2 || split_with(p->sp.N, p->prec, l, &s) != MPA_OK) return p->sp;
+    return s;
+}
+
 int adj_layout(const mpa_plan* p, double z_from, double z_to, AdjLayout* a) {
     if (p->wf) return MPA_ERR_INVALID_ARG;
     if (p->sp.logN < 13) return MPA_ERR_UNSUPPORTED_N;
@@ -56,7 +69,7 @@ int adj_layout(const mpa_plan* p, double z_from, double z_to, AdjLayout* a) {
         a->amps[(size_t)q] = p->map.amps(z0, z0 + L);
         if (a->amps[(size_t)q] >= kMaxAmpsPerInterval) return MPA_ERR_GRID;
     }
-    const Split& s = p->sp;
+    const Split s = reverse_split(p);
     const size_t N = (size_t)s.N, cs = p->csize, nodes = (size_t)p->M + 1, S = (size_t)p->n_iter;
     const bool f32 = p->prec == MPA_FP32;
     const int gc = f32 ? kca_tile_cols<float>(s.logN2) : kca_tile_cols<double>(s.logN2);
@@ -171,7 +184,7 @@ template <typename T>
 int adjoint_t(mpa_plan* p, const void* field_in, const void* grad_out, void* grad_in, const AdjLayout& a,
               unsigned char* ws, double* grad_sigma, double* grad_beta2, cudaStream_t st) {
     typedef cx<T> C;
-    const Split& s = p->sp;
+    const Split s = reverse_split(p);
     const long long N = s.N;
     const int M = p->M, S = p->n_iter, nodes = M + 1;
     const size_t NM = (size_t)nodes * (size_t)N;

@@ -120,11 +120,16 @@ template <typename T> __device__ __forceinline__ T ksq(long long kk) {
     return x * x;
 }
 
+// Tiles of the reverse column pass (KCGeom's F): 16 elements a thread from
+// 1024 points on, where 32 spill registers (844 bytes a thread; 1405 -> 1100 us
+// a launch of 2^20 x 143 nodes); 512 points are faster with 32 (860 us, 1025).
+template <typename T> __host__ __device__ constexpr int kca_tiles(int L) { return sizeof(T) == 4 && L >= 1024 ? 2 : 0; }
+
 template <typename T, int L, int MODE>
-__global__ void __launch_bounds__(KCGeom<T, L>::NT, KCGeom<T, L>::NT <= 256 && sizeof(T) == 4 ? MPA_ADJ_MINB : 1) kca_kernel(const KCAParams<T> p) {
+__global__ void __launch_bounds__(KCGeom<T, L, kca_tiles<T>(L)>::NT, KCGeom<T, L, kca_tiles<T>(L)>::NT <= 256 && sizeof(T) == 4 ? MPA_ADJ_MINB : 1) kca_kernel(const KCAParams<T> p) {
     typedef cx<T> C;
-    typedef KCGeom<T, L> Gm;
-    typedef Tiling<T> P;
+    typedef KCGeom<T, L, kca_tiles<T>(L)> Gm;
+    typedef typename Gm::P P;
     constexpr int G = Gm::G, TE = Gm::TE, NT = Gm::NT;
     constexpr bool INV = (MODE == KCA_G);
     typedef Xform<T, L, G, NT, P::RMAX, +1, LAYOUT_COL, P::PSH, true> XF;
