@@ -325,6 +325,15 @@ __device__ __forceinline__ void expi_turns_poly2(unsigned long long ta, unsigned
 }
 #endif
 
+// Element r of a run of phases: an even r evaluates the pair r, r + 1 and keeps
+// the second for the next call.
+template <int R> __device__ __forceinline__ float2 expi_pair(const unsigned long long (&th)[R], int r, float2& odd) {
+    if (r & 1) return odd;
+    float2 e;
+    expi_turns_poly2(th[r], th[r + 1], e, odd);
+    return e;
+}
+
 // (sin, cos) of a Kerr phase phi = sigma |A|^2 dz of the split-step.  These
 // phases are small (about 1e-3 rad on the benchmark links), so for
 // |phi| <= 1/16 the Taylor series of cos and sin are used: through phi^8 and

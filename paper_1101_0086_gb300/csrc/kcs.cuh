@@ -220,12 +220,17 @@ __global__ void __launch_bounds__(KCSGeom<L>::THREADS, 1)
                 const long long D = (long long)p.N1 * (L / XA::R0);
                 PhaseRun pr(c + (long long)j * p.N1 - (long long)(XA::R0 / 2) * D, D, nc);
 #pragma unroll
-                for (int u = 0; u < XA::R0; ++u) {
-                    const int r = (u + XA::R0 / 2) % XA::R0;
+                for (int u = 0; u < XA::R0; u += 2) {
+                    const int r = (u + XA::R0 / 2) % XA::R0;  // elements r, r + 1 (R0 / 2 is even)
                     const int row = j + r * (L / XA::R0);
-                    const C v = ok ? stage[row * G + g] : mkc(0.f, 0.f);
+                    const C va = ok ? stage[row * G + g] : mkc(0.f, 0.f);
+                    const C vb = ok ? stage[(row + L / XA::R0) * G + g] : mkc(0.f, 0.f);
                     // MPA step 2: A_hat_j = psi_j exp(i beta(w, z_j) + int G)
-                    vin[q][r] = cscale(cmul(v, expi_turns_poly(pr.next())), (float)nc.pre);
+                    C ea, eb;
+                    const unsigned long long ta = pr.next();
+                    expi_turns_poly2(ta, pr.next(), ea, eb);
+                    vin[q][r] = cscale(cmul(va, ea), (float)nc.pre);
+                    vin[q][r + 1] = cscale(cmul(vb, eb), (float)nc.pre);
                 }
             } else {
 #pragma unroll

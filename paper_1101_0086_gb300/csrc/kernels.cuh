@@ -257,6 +257,7 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
         unsigned long long th[XA::R0];
         if constexpr (FAST && MODE == KC_MPA_PRE)
             phase_run<XA::R0>(c + (long long)j * p.N1, (long long)p.N1 * (L / XA::R0), nc, th);
+        [[maybe_unused]] C odd = mkc(T(0), T(0));
 #pragma unroll
         for (int r = 0; r < XA::R0; ++r) {
             const int row = j + r * (L / XA::R0);
@@ -264,7 +265,7 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
             if constexpr (MODE == KC_MPA_PRE) {
                 // MPA step 2: A_hat_j = psi_j exp(i beta(w, z_j) + int G)
                 C ph;
-                if constexpr (FAST) ph = expi_turns_poly(th[r]);
+                if constexpr (FAST) ph = expi_pair(th, r, odd);
                 else ph = expi_at<T, L>(phase_q64(signed_k(c + (long long)row * p.N1, p.N), nc), thi);
                 v = cscale(cmul(v, ph), (T)nc.pre);
             }
@@ -312,11 +313,12 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
             const long long c = (col0 + g) & N1m;
             unsigned long long th[XF::RL];
             if constexpr (FAST) phase_run<XF::RL>(c + (long long)j * p.N1, (long long)p.N1 * (L / XF::RL), p.flow, th);
+        [[maybe_unused]] C odd = mkc(T(0), T(0));
 #pragma unroll
             for (int r = 0; r < XF::RL; ++r) {
                 const int row = j + r * (L / XF::RL);
                 C ph;
-                if constexpr (FAST) ph = expi_turns_poly(th[r]);
+                if constexpr (FAST) ph = expi_pair(th, r, odd);
                 else ph = expi_at<T, L>(phase_q64(signed_k(c + (long long)row * p.N1, p.N), p.flow), thi);
                 vm[q][r] = cscale(cmul(vm[q][r], ph), (T)p.flow.pre);
             }
@@ -353,6 +355,7 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
         constexpr bool HOIST = (L / RO) % Gm::OLO == 0;
         C wlo = mkc(T(1), T(0));
         if constexpr (FAC && HOIST) wlo = olo[(j & (Gm::OLO - 1)) * G + g];
+        [[maybe_unused]] C odd = mkc(T(0), T(0));
 #pragma unroll
         for (int r = 0; r < RO; ++r) {
             const int row = j + r * (L / RO);
@@ -367,7 +370,7 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
             if constexpr (MODE == KC_MPA_POST) {
                 // V_j = sigma(z_j) dz F[|A_j|^2 A_j] exp(-i beta(w, z_j) - int G)   (Eq. (6))
                 C ph;
-                if constexpr (FAST) ph = expi_turns_poly(th[r]);
+                if constexpr (FAST) ph = expi_pair(th, r, odd);
                 else ph = expi_at<T, L>(phase_q64(signed_k(c + (long long)row * p.N1, p.N), nc), thi);
                 v = cscale(cmul(v, cconj(ph)), (T)nc.post);
             }
@@ -585,12 +588,13 @@ __device__ __forceinline__ void kn_tile(const KNParams<T>& p, long long row0, un
             nc = p.nodes[p.loff[l] + jn];
         unsigned long long th[XI::R0];
         if constexpr (FAST) phase_run<XI::R0>(j, L / XI::R0, nc, th);
+        C odd = mkc(T(0), T(0));
 #pragma unroll
         for (int r = 0; r < XI::R0; ++r) {
             const int k = j + r * (L / XI::R0);
             C v = ok && MPA_DBG_OK(p.dbg, src + k, sizeof(C)) ? ldx<CG>(src + k) : mkc(T(0), T(0));
             C ph;
-            if constexpr (FAST) ph = expi_turns_poly(th[r]);
+            if constexpr (FAST) ph = expi_pair(th, r, odd);
             else ph = expi_at<T, L>(phase_q64(signed_k(k, L), nc), thi);
             vin[q][r] = cscale(cmul(v, ph), (T)nc.pre);
         }
@@ -634,11 +638,12 @@ __device__ __forceinline__ void kn_tile(const KNParams<T>& p, long long row0, un
             nc = p.nodes[p.loff[l] + jn];
         unsigned long long th[XF::RL];
         if constexpr (FAST) phase_run<XF::RL>(j, L / XF::RL, nc, th);
+        C odd = mkc(T(0), T(0));
 #pragma unroll
         for (int r = 0; r < XF::RL; ++r) {
             const int k = j + r * (L / XF::RL);
             C ph;
-            if constexpr (FAST) ph = expi_turns_poly(th[r]);
+            if constexpr (FAST) ph = expi_pair(th, r, odd);
             else ph = expi_at<T, L>(phase_q64(signed_k(k, L), nc), thi);
             if (MPA_DBG_OK(p.dbg, dst + k, sizeof(C))) dst[k] = cscale(cmul(vout[q][r], cconj(ph)), (T)nc.post);
         }
