@@ -204,7 +204,7 @@ struct Split {
     long long N, N1, N2;
     // node transforms of the MPA levels on chip (kn_kernel, one node per
     // tile row) instead of the column, row and column passes; N1 x N2 stays
-    // the split of the entry/exit transforms and of the reverse mode
+    // the split that the reverse mode starts from (reverse_split)
     bool onchip = false;
 };
 

@@ -604,7 +604,7 @@ int mpa_plan_set_split(mpa_plan* p, int32_t log2_n2) {
     if (!p) return MPA_ERR_INVALID_ARG;
     if (p->wf) return log2_n2 == p->sp.logN2 ? MPA_OK : MPA_ERR_UNSUPPORTED_N;
     if (log2_n2 == 0) {
-        // on-chip node transforms; the entry/exit transforms keep a four-step split
+        // on-chip node transforms; the reverse mode keeps a four-step split
         if (!onchip_ok(p->sp.N, p->prec)) return MPA_ERR_UNSUPPORTED_N;
         if (p->sp.onchip) return MPA_OK;
         Split s;
