@@ -154,7 +154,11 @@ cudaError_t ssr_one(const SSRParams<T>& p, cudaStream_t st) {
 
 // the tiles of field_tiles(), as the forward passes
 template <typename T, int L, int MODE> cudaError_t ssc_field(const SSCParams<T>& p, cudaStream_t st) {
-    return field_tiles<T>(L, p.N) == 1 ? ssc_one<T, L, MODE, 1>(p, st) : ssc_one<T, L, MODE, 2>(p, st);
+    const int f = field_tiles<T>(L, p.N);
+    if constexpr (L == 2048 && sizeof(T) == 4) {
+        if (f == 0) return ssc_one<T, L, MODE, 0>(p, st);
+    }
+    return f == 1 ? ssc_one<T, L, MODE, 1>(p, st) : ssc_one<T, L, MODE, 2>(p, st);
 }
 template <typename T, int L, int MODE> cudaError_t ssr_field(const SSRParams<T>& p, cudaStream_t st) {
     if constexpr (field_tiles<T>(L, 0) == 0) return ssr_one<T, L, MODE, 0>(p, st);
@@ -170,7 +174,8 @@ cudaError_t ssr_mode(int mode, const SSRParams<T>& p, cudaStream_t st) {
 }
 // columns per tile of ssc and rows per tile of ssr for a field of N samples
 template <typename T, int L> int ss_cols(long long N) {
-    return field_tiles<T>(L, N) == 1 ? KCGeom<T, L, 1>::G : KCGeom<T, L, 2>::G;
+    const int f = field_tiles<T>(L, N);
+    return f == 0 ? KCGeom<T, L>::G : f == 1 ? KCGeom<T, L, 1>::G : KCGeom<T, L, 2>::G;
 }
 template <typename T, int L> int ss_rows(long long N) {
     const int f = field_tiles<T>(L, N);

@@ -918,9 +918,13 @@ template <> struct Tiling<float, 5> {
 // so small fields need their elements spread over all of them): 2^12 244 / 71
 // / 46, 2^16 228 / 69 / 42, 2^17 221 / 70.6 / 68.4, 2^18 230 / 123 / 128, 2^20
 // 443 / 421 / 425, 2^22 1709 / 1691 / 1835.  Rows above 2048 points keep the
-// large tiles (one or a few rows each).
+// large tiles (one or a few rows each), and so do FP32 columns of 2048 points
+// beyond 2^22 (HBM-bound, 64-byte row segments against the medium tiles' 32:
+// a 2^24 step 277 against 299 us).
 template <typename T> __host__ __device__ constexpr int field_tiles(int L, long long elems) {
-    return L > 2048 ? 0 : elems <= (sizeof(T) == 8 ? 1ll << 16 : 1ll << 18) ? 1 : 2;
+    return L > 2048 || (sizeof(T) == 4 && L == 2048 && elems > (1ll << 22)) ? 0
+         : elems <= (sizeof(T) == 8 ? 1ll << 16 : 1ll << 18)               ? 1
+                                                                           : 2;
 }
 #ifndef MPA_RMAX32
 #define MPA_RMAX32 32

@@ -112,7 +112,11 @@ static cudaError_t kc_one(const KCParams<float>& pin, cudaStream_t st) {
 }
 
 template <int L, int MODE> static cudaError_t kc_field(const KCParams<float>& p, cudaStream_t st) {
-    return field_tiles<float>(L, p.ncols * L) == 1 ? kc_one<L, MODE, 1>(p, st) : kc_one<L, MODE, 2>(p, st);
+    const int f = field_tiles<float>(L, p.ncols * L);
+    if constexpr (L == 2048) {
+        if (f == 0) return kc_one<L, MODE, 0>(p, st);
+    }
+    return f == 1 ? kc_one<L, MODE, 1>(p, st) : kc_one<L, MODE, 2>(p, st);
 }
 
 template <int L>
