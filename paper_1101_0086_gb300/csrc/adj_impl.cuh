@@ -178,8 +178,8 @@ template <typename T, int L> int ss_cols(long long N) {
     return f == 0 ? KCGeom<T, L>::G : f == 1 ? KCGeom<T, L, 1>::G : KCGeom<T, L, 2>::G;
 }
 template <typename T, int L> int ss_rows(long long N) {
-    const int f = field_tiles<T>(L, N);
-    return f == 0 ? KRGeom<T, L>::G : f == 1 ? KRGeom<T, L, 1>::G : KRGeom<T, L, 2>::G;
+    if constexpr (field_tiles<T>(L, 0) == 0) return KRGeom<T, L>::G;
+    else return field_tiles<T>(L, N) == 1 ? KRGeom<T, L, 1>::G : KRGeom<T, L, 2>::G;
 }
 template <typename T> int ssc_cols_any(int logL, long long N) {
     switch (logL) {
