@@ -132,15 +132,15 @@ __global__ void __launch_bounds__(KCGeom<T, L, kca_tiles<T>(L)>::NT, KCGeom<T, L
     typedef typename Gm::P P;
     constexpr int G = Gm::G, TE = Gm::TE, NT = Gm::NT;
     constexpr bool INV = (MODE == KCA_G);
-    typedef Xform<T, L, G, NT, P::RMAX, +1, LAYOUT_COL, P::PSH, true> XF;
-    typedef Xform<T, L, G, NT, P::RMAX, -1, LAYOUT_COL, P::PSH, false> XI;
+    typedef Xform<T, L, G, NT, P::RMAX, +1, LAYOUT_COL, P::PSH, true, 0, false, Gm::EX> XF;
+    typedef Xform<T, L, G, NT, P::RMAX, -1, LAYOUT_COL, P::PSH, false, 0, false, Gm::EX> XI;
     typedef typename std::conditional<INV, XI, XF>::type XA;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[NT / 32];
     C* s = reinterpret_cast<C*>(smem_raw);
     C* thi = s + TE + (TE >> P::PSH) + 1;
     C* tlo = thi + TwDims<L>::NHI;
-    C* olo = thi + Tw<T, L>::N;
+    C* olo = thi + Tw<T, L, Gm::EX>::N;
     C* ohi = olo + G * Gm::OLO;
     const int tid = threadIdx.x;
     const long long col0 = (long long)blockIdx.x * G;
@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(KCGeom<T, L, kca_tiles<T>(L)>::NT, KCGeom<T, L
     const C* aux = p.aux + (long long)node * p.aux_stride;
     C* gn = p.g + (long long)node * p.N;
 
-    tw_init<T, L>(thi, tlo, tid, NT);
+    tw_init<T, L, Gm::EX>(thi, tlo, tid, NT);
     if constexpr (INV) {
         for (int i = tid; i < G * (Gm::OLO + Gm::OHI); i += NT) {
             const int g = i % G, m = i / G;
@@ -485,15 +485,15 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
     typedef KCGeom<T, L, F> Gm;
     typedef typename Gm::P P;
     constexpr int G = Gm::G, TE = Gm::TE, NT = Gm::NT;
-    typedef Xform<T, L, G, NT, P::RMAX, +1, LAYOUT_COL, P::PSH, true> XF;
-    typedef Xform<T, L, G, NT, P::RMAX, -1, LAYOUT_COL, P::PSH, false> XI;
+    typedef Xform<T, L, G, NT, P::RMAX, +1, LAYOUT_COL, P::PSH, true, 0, false, Gm::EX> XF;
+    typedef Xform<T, L, G, NT, P::RMAX, -1, LAYOUT_COL, P::PSH, false, 0, false, Gm::EX> XI;
     static_assert(XF::RL == XI::R0, "forward/inverse junction radix");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[NT / 32];
     C* s = reinterpret_cast<C*>(smem_raw);
     C* thi = s + TE + (TE >> P::PSH) + 1;
     C* tlo = thi + TwDims<L>::NHI;
-    C* olo = thi + Tw<T, L>::N;
+    C* olo = thi + Tw<T, L, Gm::EX>::N;
     C* ohi = olo + G * Gm::OLO;
     const int tid = threadIdx.x;
     const long long col0 = (long long)blockIdx.x * G;
@@ -501,7 +501,7 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
     constexpr bool FAST = sizeof(T) == 4;
 
     pdl_go();
-    tw_init<T, L>(thi, tlo, tid, NT);
+    tw_init<T, L, Gm::EX>(thi, tlo, tid, NT);
     for (int i = tid; i < G * (Gm::OLO + Gm::OHI); i += NT) {
         const int g = i % G, m = i / G;
         const long long k1 = (col0 + g) & N1m;
@@ -570,21 +570,21 @@ __global__ void __launch_bounds__(KRGeom<T, L, F>::NT, KRGeom<T, L, F>::NT <= 25
     typedef KRGeom<T, L, F> Gm;
     typedef typename Gm::P P;
     constexpr int G = Gm::G, TE = Gm::TE, NT = Gm::NT;
-    typedef Xform<T, L, G, NT, P::RMAX, -1, LAYOUT_ROW, P::PSH, false> XI;
-    typedef Xform<T, L, G, NT, P::RMAX, +1, LAYOUT_ROW, P::PSH, true> XF;
+    typedef Xform<T, L, G, NT, P::RMAX, -1, LAYOUT_ROW, P::PSH, false, 0, false, Gm::EX> XI;
+    typedef Xform<T, L, G, NT, P::RMAX, +1, LAYOUT_ROW, P::PSH, true, 0, false, Gm::EX> XF;
     static_assert(XI::RL == XF::R0, "inverse/forward junction radix");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[NT / 32];
     C* s = reinterpret_cast<C*>(smem_raw);
     C* thi = s + TE + (TE >> P::PSH) + 1;
     C* tlo = thi + TwDims<L>::NHI;
-    C* olo = thi + Tw<T, L>::N;
+    C* olo = thi + Tw<T, L, Gm::EX>::N;
     C* ohi = olo + G * Gm::OLO;
     const int tid = threadIdx.x;
     const long long row0 = (long long)blockIdx.x * G;
 
     pdl_go();
-    tw_init<T, L>(thi, tlo, tid, NT);
+    tw_init<T, L, Gm::EX>(thi, tlo, tid, NT);
     for (int i = tid; i < G * (Gm::OLO + Gm::OHI); i += NT) {
         const int g = i / (Gm::OLO + Gm::OHI), m = i % (Gm::OLO + Gm::OHI);
         const long long n2 = (row0 + g) & (p.N2 - 1);

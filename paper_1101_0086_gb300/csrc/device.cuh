@@ -555,10 +555,52 @@ template <int L> struct TwDims {
 // FP64 transforms of up to 2048 points keep the whole table of W_L instead
 // (hi[e], no product per lookup): FP64 instructions are the bound of the
 // FP64 passes (1.7 a clock and SM), shared-memory reads are not.
-template <typename T, int L> struct Tw {
-    static constexpr bool FULL = sizeof(T) == 8 && L >= 16 && L <= 2048;
-    static constexpr int N = FULL ? L : TwDims<L>::NLO + TwDims<L>::NHI;  // entries in shared memory
+// EX (FP32: the single-field tiles and the on-chip transforms of few nodes, up
+// to 2048 points): factors within about half a unit in the last place, since
+// passes of radix 4 to 16 apply more of them than radix-32 passes.  Split steps
+// apply the same factors at every step, so a factor's error adds up from step to
+// step where roundings of the data average out.  Error of 40 steps against FP64,
+// 2^18 samples: factors hi lo (three roundings) 1.27e-5, EX 6.7e-6 (the large
+// tiles' two radix-32 passes 1.14e-5); 2^10: 4.3e-6, 2.9e-6 (3.7e-6).  Up to 128
+// points the whole table, one lookup a factor.  From 256 on a whole table costs
+// up to 16 KB, bank conflicts and one CTA an SM less (us a step at 2^18 13.1 ->
+// 16.1, at 2^22 67 -> 85), so the two-level one holds lo - 1 instead of lo and
+// what FP32 leaves of hi = W_NHI^h (NHI <= 32): hi + (res + hi (lo - 1)), two
+// additions more than hi lo (13.6 and 68 us; 2^20 22.6 -> 23.3).
+template <typename T, int L, bool EX = false> struct Tw {
+    static constexpr bool FULL = L >= 16 && (sizeof(T) == 8 ? L <= 2048 : EX && L <= 128);
+    static constexpr bool COMP = EX && !FULL && L <= 2048;
+    static_assert(!COMP || (sizeof(T) == 4 && TwDims<L>::NHI <= 32), "hi from the table of W_32");
+    // entries in shared memory: [hi][lo][res of hi]
+    static constexpr int N = FULL ? L : TwDims<L>::NLO + (COMP ? 2 : 1) * TwDims<L>::NHI;
 };
+
+// W_32^m in FP32 and what FP32 leaves of it, from the closed forms above.
+struct W32 {
+    float2 hi[32], res[32];
+};
+template <int M> constexpr double w32_cos() {
+    if constexpr (M > 16) return w32_cos<32 - M>();
+    else if constexpr (M % 8 == 0) return M == 0 ? 1.0 : M == 8 ? 0.0 : -1.0;
+    else if constexpr (M % 4 == 0) return M == 4 ? MPA_COS_PI_4 : -MPA_COS_PI_4;
+    else return Cs32<M>::c;
+}
+template <int M = 0> constexpr void w32_fill(W32& t) {
+    if constexpr (M < 32) {
+        constexpr double c = w32_cos<M>(), s = w32_cos<(M + 24) % 32>();  // sin x = cos(x - turn / 4)
+        t.hi[M].x = (float)c;
+        t.hi[M].y = (float)s;
+        t.res[M].x = (float)(c - (double)(float)c);
+        t.res[M].y = (float)(s - (double)(float)s);
+        w32_fill<M + 1>(t);
+    }
+}
+constexpr W32 w32_make() {
+    W32 t{};
+    w32_fill(t);
+    return t;
+}
+static __constant__ const W32 kW32 = w32_make();
 
 // Slot of entry e of the low twiddle table.  A row-pass warp looks up
 // e = s j for 32 consecutive j and a power of two s; 8-byte entries sit in 16
@@ -570,9 +612,9 @@ template <int NLO> __device__ __forceinline__ int tw_lo_slot(int e) {
     else return e;
 }
 
-template <typename T, int L> __device__ __forceinline__ void tw_init(cx<T>* hi, cx<T>* lo, int tid, int nt) {
+template <typename T, int L, bool EX = false> __device__ __forceinline__ void tw_init(cx<T>* hi, cx<T>* lo, int tid, int nt) {
     typedef TwDims<L> D;
-    if constexpr (Tw<T, L>::FULL) {
+    if constexpr (Tw<T, L, EX>::FULL) {
         // the first octant evaluated, the others its reflections (exact)
         for (int m = tid; m <= L / 8; m += nt) {
             const cx<T> w = expi_ratio<T>(m, D::logL);
@@ -585,6 +627,18 @@ template <typename T, int L> __device__ __forceinline__ void tw_init(cx<T>* hi, 
             hi[3 * L / 4 + m] = mkc(w.y, -w.x);
             if (m > 0) hi[L - m] = mkc(w.x, -w.y);
         }
+    } else if constexpr (Tw<T, L, EX>::COMP) {
+        for (int i = tid; i < D::NLO + D::NHI; i += nt) {
+            if (i < D::NLO) {
+                // cos x - 1 = -2 sin^2(x/2)
+                const T h = expi_ratio<T>(i, D::logL + 1).y;
+                lo[tw_lo_slot<D::NLO>(i)] = mkc(T(-2) * h * h, expi_ratio<T>(i, D::logL).y);
+            } else {
+                const int m = i - D::NLO;
+                hi[m] = kW32.hi[m * (32 / D::NHI)];
+                lo[D::NLO + m] = kW32.res[m * (32 / D::NHI)];
+            }
+        }
     } else {
         for (int i = tid; i < D::NLO + D::NHI; i += nt) {
             if (i < D::NLO) lo[tw_lo_slot<D::NLO>(i)] = expi_ratio<T>(i, D::logL);
@@ -593,10 +647,13 @@ template <typename T, int L> __device__ __forceinline__ void tw_init(cx<T>* hi, 
     }
 }
 
-template <typename T, int L> __device__ __forceinline__ cx<T> tw_get(const cx<T>* hi, const cx<T>* lo, int e) {
+template <typename T, int L, bool EX> __device__ __forceinline__ cx<T> tw_get(const cx<T>* hi, const cx<T>* lo, int e) {
     typedef TwDims<L> D;
-    if constexpr (Tw<T, L>::FULL) return hi[e];
-    else if constexpr (D::NHI == 1) return lo[tw_lo_slot<D::NLO>(e)];
+    if constexpr (Tw<T, L, EX>::FULL) return hi[e];
+    else if constexpr (Tw<T, L, EX>::COMP) {
+        const cx<T> h = hi[e >> D::SH], l = lo[tw_lo_slot<D::NLO>(e & (D::NLO - 1))], q = lo[D::NLO + (e >> D::SH)];
+        return mkc(h.x + ffma(h.x, l.x, ffma(-h.y, l.y, q.x)), h.y + ffma(h.x, l.y, ffma(h.y, l.x, q.y)));
+    } else if constexpr (D::NHI == 1) return lo[tw_lo_slot<D::NLO>(e)];
     else return cmul(hi[e >> D::SH], lo[tw_lo_slot<D::NLO>(e & (D::NLO - 1))]);
 }
 
@@ -629,27 +686,27 @@ template <typename T, int L> __device__ __forceinline__ cx<T> expi_at(unsigned l
 // v[r] *= W_L^{S r e1} for r = 1..R-1 (R <= 32): table lookups of
 // w1, w2, w4 (combined into w1..w7) and w8, w16 (w24 = w8 w16), then
 // w_r = w_{r mod 8} w_{8 floor(r/8)}, at most three products deep.
-template <typename T, int L, int R, int S>
+template <typename T, int L, int R, int S, bool EX>
 __device__ __forceinline__ void twiddle_row(cx<T>* v, int e1, const cx<T>* hi, const cx<T>* lo) {
     typedef cx<T> C;
-    if constexpr (Tw<T, L>::FULL) {
+    if constexpr (Tw<T, L, EX>::FULL) {
 #pragma unroll
         for (int r = 1; r < R; ++r) v[r] = mul_dir<S>(v[r], hi[r * e1]);
     } else {
         C w[8];
-        w[1] = tw_get<T, L>(hi, lo, e1);
-        if constexpr (R > 2) w[2] = tw_get<T, L>(hi, lo, 2 * e1);
+        w[1] = tw_get<T, L, EX>(hi, lo, e1);
+        if constexpr (R > 2) w[2] = tw_get<T, L, EX>(hi, lo, 2 * e1);
         if constexpr (R > 2) w[3] = cmul(w[1], w[2]);
         if constexpr (R > 4) {
-            w[4] = tw_get<T, L>(hi, lo, 4 * e1);
+            w[4] = tw_get<T, L, EX>(hi, lo, 4 * e1);
             w[5] = cmul(w[1], w[4]);
             w[6] = cmul(w[2], w[4]);
             w[7] = cmul(w[3], w[4]);
         }
         C u[4];
-        if constexpr (R > 8) u[1] = tw_get<T, L>(hi, lo, 8 * e1);
+        if constexpr (R > 8) u[1] = tw_get<T, L, EX>(hi, lo, 8 * e1);
         if constexpr (R > 16) {
-            u[2] = tw_get<T, L>(hi, lo, 16 * e1);
+            u[2] = tw_get<T, L, EX>(hi, lo, 16 * e1);
             u[3] = cmul(u[1], u[2]);
         }
 #pragma unroll
@@ -692,7 +749,8 @@ template <int NS, int R, int S> __device__ __forceinline__ void dt_row(float2* v
 // read and write phases).  Butterfly j of transform g reads elements
 // j + r L/R, applies W_{NS R}^{S r (j mod NS)}, does the R-point DFT and
 // writes to (j - j mod NS) R + j mod NS + r NS.
-template <typename T, int L, int G, int NT, int R, int NS, int S, int LAYOUT, int PSH, bool SF, int GRP = 0, bool DT = false>
+template <typename T, int L, int G, int NT, int R, int NS, int S, int LAYOUT, int PSH, bool SF, int GRP = 0, bool DT = false,
+          bool EX = false>
 __device__ __forceinline__ void stockham_pass(cx<T>* s, const cx<T>* hi, const cx<T>* lo, const cx<T>* dt = nullptr) {
     typedef cx<T> C;
     constexpr int NB = (L / R) * G;
@@ -714,7 +772,7 @@ __device__ __forceinline__ void stockham_pass(cx<T>* s, const cx<T>* hi, const c
             for (int r = 0; r < R; ++r) v[q][r] = s[phys<PSH>(eidx<LAYOUT, L, G>(j + r * (L / R), g))];
         }
         if constexpr (DT) dt_row<NS, R, S>(v[q], dt, j & (NS - 1));
-        else if constexpr (NS > 1) twiddle_row<T, L, R, S>(v[q], (j & (NS - 1)) * (L / (NS * R)), hi, lo);
+        else if constexpr (NS > 1) twiddle_row<T, L, R, S, EX>(v[q], (j & (NS - 1)) * (L / (NS * R)), hi, lo);
         Dft<R, S, C>::run(v[q]);
     }
     gsync<GRP, NT>();
@@ -758,13 +816,13 @@ template <int L, int RMAX> struct Sched {
     template <bool SF> __host__ __device__ static constexpr int ns(int p) { return p == 0 ? 1 : ns<SF>(p - 1) * radix<SF>(p - 1); }
 };
 
-template <typename T, int L, int G, int NT, int RMAX, int S, int LAYOUT, int PSH, bool SF, int P, int NP, int GRP, bool DT>
+template <typename T, int L, int G, int NT, int RMAX, int S, int LAYOUT, int PSH, bool SF, int P, int NP, int GRP, bool DT, bool EX>
 __device__ __forceinline__ void mid_passes(cx<T>* s, const cx<T>* hi, const cx<T>* lo, const cx<T>* dt) {
     if constexpr (P < NP - 1) {
         typedef Sched<L, RMAX> SC;
         stockham_pass<T, L, G, NT, SC::template radix<SF>(P), SC::template ns<SF>(P), S, LAYOUT, PSH, SF, GRP,
-                      DT && P == 1>(s, hi, lo, dt);
-        mid_passes<T, L, G, NT, RMAX, S, LAYOUT, PSH, SF, P + 1, NP, GRP, DT>(s, hi, lo, dt);
+                      DT && P == 1, EX>(s, hi, lo, dt);
+        mid_passes<T, L, G, NT, RMAX, S, LAYOUT, PSH, SF, P + 1, NP, GRP, DT, EX>(s, hi, lo, dt);
     }
 }
 
@@ -785,8 +843,10 @@ template <int LAYOUT, int L, int G, int R> __host__ __device__ __forceinline__ v
 // used by the middle passes only; the transform ends with a barrier so the
 // caller may reuse `s`.  GRP as for gtid/gsync.  USE_DT: the second pass reads
 // its twiddles from a direct table of DTN entries (where that is at most 1024;
-// 0: none) that the caller fills with dt_init and passes to run.
-template <typename T, int L, int G, int NT, int RMAX, int S, int LAYOUT, int PSH, bool SF, int GRP = 0, bool USE_DT = false>
+// 0: none) that the caller fills with dt_init and passes to run.  EX: the
+// factors of Tw's EX tables.
+template <typename T, int L, int G, int NT, int RMAX, int S, int LAYOUT, int PSH, bool SF, int GRP = 0, bool USE_DT = false,
+          bool EX = false>
 struct Xform {
     typedef Sched<L, RMAX> SC;
     typedef cx<T> C;
@@ -846,7 +906,7 @@ struct Xform {
             }
             gsync<GRP, NT>();
             hook();
-            mid_passes<T, L, G, NT, RMAX, S, LAYOUT, PSH, SF, 1, NP, GRP, DT>(s, hi, lo, dt);
+            mid_passes<T, L, G, NT, RMAX, S, LAYOUT, PSH, SF, 1, NP, GRP, DT, EX>(s, hi, lo, dt);
             // last pass (NS = L/RL, so k = j): gather j + r L/RL, twiddle W_L^{S r j}, DFT
 #pragma unroll
             for (int q = 0; q < QL; ++q) {
@@ -862,7 +922,7 @@ struct Xform {
                     for (int r = 0; r < RL; ++r) vout[q][r] = s[phys<PSH>(eidx<LAYOUT, L, G>(j + r * (L / RL), g))];
                 }
                 if constexpr (DT && NP == 2) dt_row<NS1, R1, S>(vout[q], dt, j);
-                else twiddle_row<T, L, RL, S>(vout[q], j, hi, lo);
+                else twiddle_row<T, L, RL, S, EX>(vout[q], j, hi, lo);
                 Dft<RL, S, C>::run(vout[q]);
             }
             gsync<GRP, NT>();

@@ -114,13 +114,14 @@ template <typename T> struct KRParams {
 // F: the tiles of field_tiles().
 template <typename T, int L, int F = 0> struct KCGeom {
     typedef Tiling<T, F ? F + 2 : 0> P;
+    static constexpr bool EX = F > 0 && sizeof(T) == 4;  // FP32 single fields: Tw's EX tables
     static constexpr int G = (P::TE / L) > P::CMIN ? (P::TE / L) : P::CMIN;
     static constexpr int TE = G * L;
     static constexpr int NT = TE / P::E;
     static constexpr int OSH = 5;  // outer-factor two-level split of n2
     static constexpr int OLO = L < 32 ? L : 32;
     static constexpr int OHI = L > 32 ? L / 32 : 1;
-    static constexpr size_t smem_elems = (size_t)TE + (TE >> P::PSH) + 1 + Tw<T, L>::N +
+    static constexpr size_t smem_elems = (size_t)TE + (TE >> P::PSH) + 1 + Tw<T, L, EX>::N +
                                          (size_t)G * (OLO + OHI);
     // FP32: + the exp(2 pi i m/1024) table of the per-element phases
     static constexpr size_t smem_bytes = smem_elems * sizeof(cx<T>);
@@ -128,13 +129,14 @@ template <typename T, int L, int F = 0> struct KCGeom {
 
 template <typename T, int L, int F = 0> struct KRGeom {
     typedef Tiling<T, F ? F + 2 : 1> P;
+    static constexpr bool EX = F > 0 && sizeof(T) == 4;
     static constexpr int G = (P::TE / L) > 1 ? (P::TE / L) : 1;
     static constexpr int TE = G * L;
     static constexpr int NT = TE / P::E;
     static constexpr int OSH = 7;  // outer-factor split of k1
     static constexpr int OLO = L < 128 ? L : 128;
     static constexpr int OHI = L > 128 ? L / 128 : 1;
-    static constexpr size_t smem_elems = (size_t)TE + (TE >> P::PSH) + 1 + Tw<T, L>::N +
+    static constexpr size_t smem_elems = (size_t)TE + (TE >> P::PSH) + 1 + Tw<T, L, EX>::N +
                                          (size_t)G * (OLO + OHI);
     static constexpr size_t smem_bytes = smem_elems * sizeof(cx<T>);
 };
@@ -204,15 +206,15 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
     constexpr bool FAC = (INV || MODE == KC_FWDF) && !ROWS;        // outer factor at the store
     // forward: small radix first, so it ends with an RMAX pass that meets the
     // inverse's first RMAX pass in registers (split-step column pass)
-    typedef Xform<T, L, G, NT, P::RMAX, +1, LAYOUT_COL, P::PSH, true> XF;
-    typedef Xform<T, L, G, NT, P::RMAX, -1, LAYOUT_COL, P::PSH, false> XI;
+    typedef Xform<T, L, G, NT, P::RMAX, +1, LAYOUT_COL, P::PSH, true, 0, false, Gm::EX> XF;
+    typedef Xform<T, L, G, NT, P::RMAX, -1, LAYOUT_COL, P::PSH, false, 0, false, Gm::EX> XI;
     static_assert(!(FWD && INV) || XF::RL == XI::R0, "forward/inverse junction radix");
     typedef typename std::conditional<FWD, XF, XI>::type XA;  // first transform
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* s = reinterpret_cast<C*>(smem_raw);
     C* thi = s + TE + (TE >> P::PSH) + 1;
     C* tlo = thi + TwDims<L>::NHI;
-    C* olo = thi + Tw<T, L>::N;  // [OLO][G]
+    C* olo = thi + Tw<T, L, Gm::EX>::N;  // [OLO][G]
     C* ohi = olo + G * Gm::OLO;     // [OHI][G]
     const int tid = threadIdx.x;
     const long long col0 = (long long)blockIdx.x * G;
@@ -222,7 +224,7 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
     // passes that a scan follows let it start only at their end (pdl_go)
     constexpr bool EARLY = F > 0 || MODE == KC_MPA_PRE || MODE == KC_INV;
     if constexpr (EARLY) pdl_go();
-    tw_init<T, L>(thi, tlo, tid, NT);
+    tw_init<T, L, Gm::EX>(thi, tlo, tid, NT);
     if constexpr (FAC) {
         // W_N^{-n2 k1} for the tile's columns: olo[m][g] = W^{-k1 m}, ohi[h][g] = W^{-k1 32 h} (FWDF: +)
         for (int i = tid; i < G * (Gm::OLO + Gm::OHI); i += NT) {
@@ -391,21 +393,21 @@ __global__ void __launch_bounds__(KRGeom<T, L, F>::NT, KRGeom<T, L, F>::NT <= 25
     constexpr bool FWD = (MODE != KR_INV);
     // inverse: small radix last, forward: small radix first, so the two meet
     // in registers around the pointwise step
-    typedef Xform<T, L, G, NT, P::RMAX, -1, LAYOUT_ROW, P::PSH, false> XI;
-    typedef Xform<T, L, G, NT, P::RMAX, +1, LAYOUT_ROW, P::PSH, true> XF;
+    typedef Xform<T, L, G, NT, P::RMAX, -1, LAYOUT_ROW, P::PSH, false, 0, false, Gm::EX> XI;
+    typedef Xform<T, L, G, NT, P::RMAX, +1, LAYOUT_ROW, P::PSH, true, 0, false, Gm::EX> XF;
     static_assert(!(FWD && INV) || XI::RL == XF::R0, "inverse/forward junction radix");
     typedef typename std::conditional<INV, XI, XF>::type XA;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* s = reinterpret_cast<C*>(smem_raw);
     C* thi = s + TE + (TE >> P::PSH) + 1;
     C* tlo = thi + TwDims<L>::NHI;
-    C* olo = thi + Tw<T, L>::N;  // [G][OLO]
+    C* olo = thi + Tw<T, L, Gm::EX>::N;  // [G][OLO]
     C* ohi = olo + G * Gm::OLO;     // [G][OHI]
     const int tid = threadIdx.x;
     const long long row0 = (long long)blockIdx.x * G;
 
     pdl_go();
-    tw_init<T, L>(thi, tlo, tid, NT);
+    tw_init<T, L, Gm::EX>(thi, tlo, tid, NT);
     if constexpr (FWD) {
         // W_N^{+n2 k1} for the tile's rows: olo[g][m] = W^{n2 m}, ohi[g][h] = W^{n2 128 h}
         for (int i = tid; i < G * (Gm::OLO + Gm::OHI); i += NT) {
@@ -540,8 +542,9 @@ template <typename T> struct KNParams {
 template <typename T, int L, int F = 0> struct KNGeom {
     typedef KRGeom<T, L> R;
     typedef Tiling<T, F ? 5 : 1> P;
+    static constexpr bool EX = F > 0 && sizeof(T) == 4 && L <= 2048;
     static constexpr int G = F ? (L >= 1024 ? 1 : 1024 / L) : R::G, TE = G * L, NT = TE / P::E;
-    static constexpr size_t smem_bytes = ((size_t)TE + (TE >> P::PSH) + 1 + Tw<T, L>::N) * sizeof(cx<T>);
+    static constexpr size_t smem_bytes = ((size_t)TE + (TE >> P::PSH) + 1 + Tw<T, L, EX>::N) * sizeof(cx<T>);
 };
 
 // The node rows row0 .. row0 + G - 1 of a launch (one tile) through steps
@@ -552,8 +555,8 @@ __device__ __forceinline__ void kn_tile(const KNParams<T>& p, long long row0, un
     typedef KNGeom<T, L, F> Gm;
     typedef typename Gm::P P;
     constexpr int G = Gm::G, NT = Gm::NT, TE = Gm::TE;
-    typedef Xform<T, L, G, NT, P::RMAX, -1, LAYOUT_ROW, P::PSH, false> XI;
-    typedef Xform<T, L, G, NT, P::RMAX, +1, LAYOUT_ROW, P::PSH, true> XF;
+    typedef Xform<T, L, G, NT, P::RMAX, -1, LAYOUT_ROW, P::PSH, false, 0, false, Gm::EX> XI;
+    typedef Xform<T, L, G, NT, P::RMAX, +1, LAYOUT_ROW, P::PSH, true, 0, false, Gm::EX> XF;
     static_assert(XI::RL == XF::R0, "inverse/forward junction radix");
     constexpr bool FAST = sizeof(T) == 4;  // FP32: finite-difference phases + polynomial exp
     C* s = reinterpret_cast<C*>(smem_raw);
@@ -561,7 +564,7 @@ __device__ __forceinline__ void kn_tile(const KNParams<T>& p, long long row0, un
     C* tlo = thi + TwDims<L>::NHI;
     const int tid = threadIdx.x;
 
-    tw_init<T, L>(thi, tlo, tid, NT);
+    tw_init<T, L, Gm::EX>(thi, tlo, tid, NT);
     __syncthreads();
     if constexpr (!CG) pdl_wait();  // CG: called inside the persistent kernel
 
