@@ -164,7 +164,7 @@ int forward_ckpt(mpa_plan* p, const void* field, const AdjLayout& a, double2* ck
     cx<T>* psi = reinterpret_cast<cx<T>*>(p->ws + p->off_psi);
     double2* state = reinterpret_cast<double2*>(p->ws + p->off_state);
     cx<T>* psi0c = reinterpret_cast<cx<T>*>(p->ws + p->off_psi0c);
-    int rc = fft_forward<T>(s.N, reinterpret_cast<const cx<T>*>(field), psi, psi + s.N, st);
+    int rc = fft_forward<T>(s.N, reinterpret_cast<const cx<T>*>(field), psi, psi + s.N, st, &s);
     if (rc) return rc;
     MPA_TRY(to_state_launch<T>(psi, state, sizeof(T) == 4 ? psi0c : nullptr, s.N, st));
     for (long q = 0; q < a.n_int; ++q) {
@@ -175,7 +175,7 @@ int forward_ckpt(mpa_plan* p, const void* field, const AdjLayout& a, double2* ck
     MPA_TRY(cudaMemcpyAsync(ck + (size_t)a.n_int * N, state, N * sizeof(double2), cudaMemcpyDeviceToDevice, st));
     if (out) {
         MPA_TRY(from_state_launch<T>(state, psi, s.N, st));
-        return fft_inverse<T>(s.N, psi, reinterpret_cast<cx<T>*>(out), psi, st);
+        return fft_inverse<T>(s.N, psi, reinterpret_cast<cx<T>*>(out), psi, st, &s);
     }
     return MPA_OK;
 }
@@ -215,7 +215,7 @@ int adjoint_t(mpa_plan* p, const void* field_in, const void* grad_out, void* gra
     MPA_TRY(cudaMemcpyAsync(adjc, tab.data(), tab.size() * sizeof(AdjC), cudaMemcpyHostToDevice, st));
     MPA_TRY(cudaMemsetAsync(acc, 0, (size_t)a.n_int * a.acc_stride * sizeof(double), st));
     // A_out = F^-1[A_hat]  =>  g_{A_hat} = F[g_out] / N
-    int rc = fft_forward<T>(N, reinterpret_cast<const C*>(grad_out), G, G + N, st);
+    int rc = fft_forward<T>(N, reinterpret_cast<const C*>(grad_out), G, G + N, st, &p->sp);
     if (rc) return rc;
     MPA_TRY(scale_to_state_launch<T>(G, gx, 1.0 / (double)N, N, st));
 

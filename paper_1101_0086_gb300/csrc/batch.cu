@@ -157,7 +157,7 @@ int run_group(mpa_batch* b, Group& g, cudaStream_t st) {
     for (int i = 0; i < n; ++i) {
         cx<T>* scratch = psi + (long long)i * (M + 1) * N;
         int rc = fft_forward<T>(N, reinterpret_cast<const cx<T>*>(b->links[(size_t)g.links[(size_t)i]].field), scratch,
-                                scratch + N, st);
+                                scratch + N, st, &s);
         if (rc) return rc;
         MPA_TRY(to_state_launch<T>(scratch, state + (long long)i * N, sizeof(T) == 4 ? psi0c + (long long)i * N : nullptr,
                                    N, st));
@@ -177,7 +177,8 @@ int run_group(mpa_batch* b, Group& g, cudaStream_t st) {
     for (int i = 0; i < n; ++i) {
         cx<T>* scratch = psi + (long long)i * (M + 1) * N;
         MPA_TRY(from_state_launch<T>(state + (long long)i * N, scratch, N, st));
-        int rc = fft_inverse<T>(N, scratch, reinterpret_cast<cx<T>*>(b->links[(size_t)g.links[(size_t)i]].field), scratch, st);
+        int rc = fft_inverse<T>(N, scratch, reinterpret_cast<cx<T>*>(b->links[(size_t)g.links[(size_t)i]].field), scratch,
+                                st, &s);
         if (rc) return rc;
     }
     return MPA_OK;

@@ -254,9 +254,16 @@ inline int split_n(long long N, int prec, Split* s) {
 // length-N1 transforms over b at every m2, whose column-pass form (KC_FWD_T,
 // KC_INV_T) stores m2 + N2 m1, natural order again.  The split is the transform's
 // own (split_n).  Beyond 2^22 samples the second length exceeds the column
-// pass: then the field is transposed around a row pass.  The transpose and the
-// copy back that this saves were two of four launches (2^12 to 2^18 28 -> 18 us a
-// call, 2^20 37 -> 28, FP64 2^18 80 -> 65).
+// pass: then the field is transposed around a row pass, at the plan's split
+// where there is one (2^14 x 2^10 takes one pass less than 2^13 x 2^11: error of
+// a transform pair of 2^24 samples 3.6e-7, 4.8e-7).  The transpose and the copy
+// back that the two passes save were two of four launches (2^12 to 2^18 28 ->
+// 18 us a call, 2^20 37 -> 28, FP64 2^18 80 -> 65).
+template <typename T> inline int fft_split(long long N, const Split* plan, Split* s) {
+    const int rc = split_n(N, sizeof(T) == 4 ? MPA_FP32 : MPA_FP64, s);
+    if (rc == MPA_OK && plan && s->logN1 > KC_LOG_MAX) *s = *plan;
+    return rc;
+}
 template <typename T> inline KCParams<T> fft_cols(const cx<T>* src, cx<T>* dst, const Split& s, long long ncols, int log_cols) {
     KCParams<T> c{};
     c.src = src;
@@ -270,11 +277,13 @@ template <typename T> inline KCParams<T> fft_cols(const cx<T>* src, cx<T>* dst, 
 }
 
 // Forward: natural A(t) in `data` -> natural spectrum in `out` (may be
-// `data`), through `tmp` (neither of them).
+// `data`), through `tmp` (neither of them).  plan: a plan's split, where there
+// is one.
 template <typename T>
-inline int fft_forward(long long N, const cx<T>* data, cx<T>* out, cx<T>* tmp, cudaStream_t st) {
+inline int fft_forward(long long N, const cx<T>* data, cx<T>* out, cx<T>* tmp, cudaStream_t st,
+                       const Split* plan = nullptr) {
     Split s;
-    const int rc = split_n(N, sizeof(T) == 4 ? MPA_FP32 : MPA_FP64, &s);
+    const int rc = fft_split<T>(N, plan, &s);
     if (rc) return rc;
     if (s.logN1 <= KC_LOG_MAX) {
         MPA_TRY(kc_launch<T>(KC_FWDF, s.logN2, fft_cols<T>(data, tmp, s, s.N1, s.logN1), st));
@@ -291,9 +300,10 @@ inline int fft_forward(long long N, const cx<T>* data, cx<T>* out, cx<T>* tmp, c
 // Inverse: natural spectrum in `spec` -> natural A(t) in `out` (may be `spec`),
 // through `tmp` (may be `spec`, not `out`).
 template <typename T>
-inline int fft_inverse(long long N, const cx<T>* spec, cx<T>* out, cx<T>* tmp, cudaStream_t st) {
+inline int fft_inverse(long long N, const cx<T>* spec, cx<T>* out, cx<T>* tmp, cudaStream_t st,
+                       const Split* plan = nullptr) {
     Split s;
-    const int rc = split_n(N, sizeof(T) == 4 ? MPA_FP32 : MPA_FP64, &s);
+    const int rc = fft_split<T>(N, plan, &s);
     if (rc) return rc;
     MPA_TRY(kc_launch<T>(KC_INV, s.logN2, fft_cols<T>(spec, tmp, s, s.N1, s.logN1), st));
     if (s.logN1 <= KC_LOG_MAX) {

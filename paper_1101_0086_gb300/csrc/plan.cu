@@ -360,7 +360,7 @@ int propagate_t(mpa_plan* p, void* field, double z_from, double z_to, cudaStream
     double2* state = reinterpret_cast<double2*>(p->ws + p->off_state);
     cx<T>* psi0c = reinterpret_cast<cx<T>*>(p->ws + p->off_psi0c);
     // A_hat(z_from) = F[A] -> FP64 state and its working copy
-    int rc = fft_forward<T>(s.N, f, psi, psi + s.N, st);
+    int rc = fft_forward<T>(s.N, f, psi, psi + s.N, st, &s);
     if (rc) return rc;
     MPA_TRY(to_state_launch<T>(psi, state, sizeof(T) == 4 ? psi0c : nullptr, s.N, st));
     for (long q = 0; q < n_int; ++q) {
@@ -372,7 +372,7 @@ int propagate_t(mpa_plan* p, void* field, double z_from, double z_to, cudaStream
     }
     // A(z_to) = F^-1[A_hat]
     MPA_TRY(from_state_launch<T>(state, psi, s.N, st));
-    return fft_inverse<T>(s.N, psi, f, psi, st);
+    return fft_inverse<T>(s.N, psi, f, psi, st, &s);
 }
 
 template <typename T>
