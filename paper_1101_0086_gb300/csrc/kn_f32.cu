@@ -35,13 +35,16 @@ static cudaError_t kn_one(const KNParams<float>& p, cudaStream_t st) {
 // large / fine: 143 nodes 2^8 14.2 / 8.6, 2^10 13.3 / 10.1, 2^12 15.7 / 11.5, 2^13
 // 16.4 / 17.2, 2^14 19.6 / 22.7; 801 nodes 2^11 (201 tiles) 22.6 / 18.4, 2^12
 // (401 tiles) 31.7 / 32.7.
-template <int L> static bool kn_fine(const KNParams<float>& p) {
-    return (p.nrows + KNGeom<float, L>::G - 1) / KNGeom<float, L>::G < 2 * 152;
+template <int L> static bool kn_fine(const KNParams<float>& p, int sms) {
+    return !fills_twice((p.nrows + KNGeom<float, L>::G - 1) / KNGeom<float, L>::G, sms);
 }
 
 template <int L, bool PIN, bool POUT> static cudaError_t kn_any(const KNParams<float>& p, cudaStream_t st) {
     if constexpr (L <= 4096) {
-        if (kn_fine<L>(p)) return kn_one<L, PIN, POUT, 1>(p, st);
+        int sms = 0;
+        const cudaError_t e = sm_count(&sms);
+        if (e != cudaSuccess) return e;
+        if (kn_fine<L>(p, sms)) return kn_one<L, PIN, POUT, 1>(p, st);
     }
     return kn_one<L, PIN, POUT, 0>(p, st);
 }

@@ -24,9 +24,8 @@ static cudaError_t krs_one(const KRParams<float>& p, cudaStream_t st) {
     if (ea != cudaSuccess) return ea;
     const long long ntiles = (p.nrows + KRGeom<float, L>::G - 1) / KRGeom<float, L>::G;
     if (ntiles <= 0) return cudaSuccess;
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int sms = 0;
+    const cudaError_t e = sm_count(&sms);
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)(ntiles < sms ? ntiles : sms);  // one CTA per SM
     const bool prof = g_prof_on.load(std::memory_order_relaxed);

@@ -44,6 +44,21 @@ template <class F> inline cudaError_t attrs_once(AttrOnce& once, F&& set) {
     return e;
 }
 
+// SMs of the current device, asked for once a device (devices 0..63).
+inline cudaError_t sm_count(int* sms) {
+    static std::atomic<int> known[64];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const bool keep = dev >= 0 && dev < 64;
+    if (keep && (*sms = known[dev].load(std::memory_order_relaxed)) > 0) return cudaSuccess;
+    e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess && keep) known[dev].store(*sms, std::memory_order_relaxed);
+    return e;
+}
+// Whether `blocks` blocks fill `sms` SMs twice over.
+inline bool fills_twice(long long blocks, int sms) { return blocks >= 2ll * sms; }
+
 // Launch of a kernel that calls pdl_wait() before its first global access
 // (device.cuh): its launch and preparation overlap the end of the kernel
 // before it in the stream.  Split step of 2^14 modes (two kernels whose tables
@@ -66,9 +81,12 @@ inline cudaError_t launch_pdl(bool early, void (*kernel)(P...), dim3 grid, dim3 
 }
 // Whether a level's kernel of `blocks` blocks starts early: a grid that does
 // not fill the SMs twice over would be packed onto the first ones that fall
-// free (one span of a 2^12 link, 72 blocks of node transforms and 128 of the
-// scan: 761 us with ordinary launches, 861 to 940 with early ones).
-inline bool pdl_fills(long long blocks) { return blocks >= 2 * 152; }
+// free (one span of a 2^12 link, 72 blocks of two node transforms and 128 of
+// the scan: 761 us with ordinary launches, 861 to 940 with early ones).
+inline bool pdl_fills(long long blocks) {
+    int sms = 0;
+    return sm_count(&sms) == cudaSuccess && fills_twice(blocks, sms);
+}
 // Whether a pass over a single field of n samples starts early.  FP64 passes of
 // 2^16 .. 2^18 samples, bound by the schedulers they spread over, would be
 // packed too: us a split step, early / ordinary: 2^14 27 / 46, 2^15 31 / 43,

@@ -1,0 +1,22 @@
+"""Launch rules of the library (launch.h) compiled as host code by nvcc and
+checked without a GPU: which grids count as filling the device's SMs."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+def test_launch_rules(tmp_path):
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not available")
+    exe = str(tmp_path / "launch_rules_check")
+    src = os.path.join(ROOT, "tests", "native", "launch_rules_check.cu")
+    inc = os.path.join(ROOT, "paper_1101_0086_gb300", "csrc")
+    subprocess.run([nvcc, "-std=c++17", "-O2", "-gencode", "arch=compute_103a,code=sm_103a", "-I", inc, src, "-o", exe],
+                   check=True, capture_output=True, timeout=600)
+    r = subprocess.run([exe], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr
