@@ -22,9 +22,19 @@ static cudaError_t kc_one(const KCParams<double>& pin, cudaStream_t st) {
     if (ea != cudaSuccess) return ea;
     const long long nblk = (p.ncols + Gm::G - 1) / Gm::G;
     if (nblk <= 0) return cudaSuccess;
+    bool early;
+    if constexpr (F == 0) {
+        int sms = 0;
+        const cudaError_t es = sm_count(&sms);
+        if (es != cudaSuccess) return es;
+        early = pdl_level64(pair_fits(Gm::smem_bytes), nblk, sms);
+    } else {
+        early = pdl_field<double>(p.N, MODE == KC_FWDF || MODE == KC_FWD_T || MODE == KC_INV || MODE == KC_INV_T);
+    }
     const bool prof = g_prof_on.load(std::memory_order_relaxed);
     if (prof) prof_begin(st);
-    const cudaError_t el = launch_pdl(F == 0 || pdl_field<double>(p.N), kc_kernel<double, L, MODE, F>, (unsigned)nblk, Gm::NT, Gm::smem_bytes, st, p);
+    const cudaError_t el =
+        launch_pdl(early, kc_kernel<double, L, MODE, F>, (unsigned)nblk, Gm::NT, Gm::smem_bytes, st, p);
     if (prof) {
         // algorithmic bytes: every tile element read once and written once
         // (a shared source, src_stride == 0, is read once for all nodes)

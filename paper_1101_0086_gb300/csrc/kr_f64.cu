@@ -19,9 +19,19 @@ static cudaError_t kr_one(const KRParams<double>& p, cudaStream_t st) {
     if (ea != cudaSuccess) return ea;
     const long long nblk = (p.nrows + Gm::G - 1) / Gm::G;
     if (nblk <= 0) return cudaSuccess;
+    bool early;
+    if constexpr (F == 0) {
+        int sms = 0;
+        const cudaError_t es = sm_count(&sms);
+        if (es != cudaSuccess) return es;
+        early = pdl_level64(pair_fits(Gm::smem_bytes), nblk, sms);
+    } else {
+        early = pdl_field<double>(p.N);
+    }
     const bool prof = g_prof_on.load(std::memory_order_relaxed);
     if (prof) prof_begin(st);
-    const cudaError_t el = launch_pdl(F == 0 || pdl_field<double>(p.N), kr_kernel<double, L, MODE, F>, (unsigned)nblk, Gm::NT, Gm::smem_bytes, st, p);
+    const cudaError_t el =
+        launch_pdl(early, kr_kernel<double, L, MODE, F>, (unsigned)nblk, Gm::NT, Gm::smem_bytes, st, p);
     if (prof) prof_end(prof_kr_kind(MODE), st, 2.0 * (double)p.nrows * L * sizeof(cx<double>));
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return el;

@@ -87,12 +87,29 @@ inline bool pdl_fills(long long blocks) {
     int sms = 0;
     return sm_count(&sms) == cudaSuccess && fills_twice(blocks, sms);
 }
+// Whether two CTAs with `smem` bytes of shared memory each fit an SM (228 KB, 1
+// KB of them reserved for each).
+constexpr bool pair_fits(size_t smem) { return 2 * (smem + 1024) <= 228 * 1024; }
+// Whether an FP64 column or row pass of a level starts early.  Where two of its
+// CTAs fit an SM (`pair`) and it has at most one for each SM, an early start
+// packs them in pairs onto half of the SMs, and an FP64 CTA takes as long as the
+// SM's FP64 pipe has work.  A level of 143 nodes, early / ordinary: 2^12 (143
+// blocks a column pass) 415 / 293 us, 2^11 with columns of 64 (72 blocks) 268 /
+// 236.  CTAs that get an SM each in any case lose only the overlap by an ordinary
+// launch (2^10, columns of 32: 237 / 315; 2^13, 286 blocks: 560 / 569), and the
+// overlap is worth more than the packing of a few (2^10 with columns of 64, 36
+// blocks: 210 / 224).
+inline bool pdl_level64(bool pair, long long blocks, int sms) { return !pair || 4 * blocks <= sms || blocks > sms; }
 // Whether a pass over a single field of n samples starts early.  FP64 passes of
 // 2^16 .. 2^18 samples, bound by the schedulers they spread over, would be
 // packed too: us a split step, early / ordinary: 2^14 27 / 46, 2^15 31 / 43,
-// 2^16 86 / 42, 2^17 157 / 68, 2^18 189 / 123, 2^20 412 / 419; FP32: 2^14 6.2 /
-// 13.9, 2^18 12.9 / 13.8, 2^20 23.3 / 23.2, 2^22 66 / 71.
-template <typename T> inline bool pdl_field(long long n) { return sizeof(T) == 4 || n <= (1ll << 15) || n > (1ll << 18); }
+// 2^16 86 / 42, 2^17 157 / 68, 2^18 189 / 123, 2^19 230 / 237, 2^20 412 / 419;
+// FP32: 2^14 6.2 / 13.9, 2^18 12.9 / 13.8, 2^20 23.3 / 23.2, 2^22 66 / 71.  The
+// two passes of a transform of 2^19 samples are packed as well: 127 / 99 (2^20
+// 173 / 180).
+template <typename T> inline bool pdl_field(long long n, bool transform = false) {
+    return sizeof(T) == 4 || n <= (1ll << 15) || n > (1ll << (transform ? 19 : 18));
+}
 
 // Optional CUDA-event timing of every launch, by kernel kind (off by
 // default; enabled through mpa_profile).

@@ -1,5 +1,6 @@
 """Launch rules of the library (launch.h) compiled as host code by nvcc and
-checked without a GPU: which grids count as filling the device's SMs."""
+checked without a GPU: which grids count as filling the device's SMs, and which
+launches start while the kernel before them ends."""
 import os
 import shutil
 import subprocess
