@@ -77,7 +77,9 @@ inline cudaError_t launch_pdl(bool early, void (*kernel)(P...), dim3 grid, dim3 
     a.val.programmaticStreamSerializationAllowed = 1;
     c.attrs = &a;
     c.numAttrs = early ? 1 : 0;
-    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();  // returned here, not left for a later check of another call's
+    return e;
 }
 // Whether a level's kernel of `blocks` blocks starts early: a grid that does
 // not fill the SMs twice over would be packed onto the first ones that fall
