@@ -71,6 +71,11 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)), "l"(f2_bits(c)));
     return f2_from(r);
 }
+#else
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return make_float2(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y)); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    return make_float2(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y));
+}
 #endif
 template <class C> __device__ __forceinline__ C cmul(C a, C b) {
     return mkc(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -299,7 +304,6 @@ __device__ __forceinline__ float2 expi_turns_poly(unsigned long long th) {
     return make_float2(__uint_as_float(__float_as_uint(a) ^ neg), __uint_as_float(__float_as_uint(b) ^ neg));
 }
 
-#if MPA_F32X2
 // expi_turns_poly of two phases at once: the same operations, the series of
 // both phases in the two lanes of packed instructions, and the quarter turn
 // taken from the bits of theta + 1/8 turn (bit 31 of its high word: half a
@@ -323,7 +327,6 @@ __device__ __forceinline__ void expi_turns_poly2(unsigned long long ta, unsigned
     ea = make_float2(__uint_as_float(__float_as_uint(ax) ^ na), __uint_as_float(__float_as_uint(ay) ^ na));
     eb = make_float2(__uint_as_float(__float_as_uint(bx) ^ nb), __uint_as_float(__float_as_uint(by) ^ nb));
 }
-#endif
 
 // Element r of a run of phases: an even r evaluates the pair r, r + 1 and keeps
 // the second for the next call.
