@@ -610,7 +610,7 @@ static __constant__ const W32 kW32 = w32_make();
 // bank pairs, so in natural order the stride s = 4, 8, 16 lookups would
 // collide 4- to 8-fold.  XOR-ing the entry's 16-block index into its low
 // four bits spreads every such stride over distinct bank pairs.
-template <int NLO> __device__ __forceinline__ int tw_lo_slot(int e) {
+template <int NLO> __host__ __device__ __forceinline__ int tw_lo_slot(int e) {
     if constexpr (NLO >= 32) return e ^ ((e >> 4) & 15);
     else return e;
 }

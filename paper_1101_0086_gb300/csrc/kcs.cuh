@@ -33,7 +33,8 @@ template <int L> struct KCSTile {
 
 // Shared-memory layout: the stage (TE elements, row-major L x G), two
 // mbarriers, four slots of node constants (those of CTA-local tile i in
-// slot i mod 4, copied with the tile), the twiddle tables of both groups,
+// slot i mod 4, copied with the tile and read with it), the twiddle tables of
+// both groups,
 // then per group its exchange buffer and outer-factor tables.
 // Direct twiddle tables (dt_fill) in the inverse passes, which multiply
 // second passes of radix 32, 16 and 8 by them (1024 points: 462 -> 442 us a
