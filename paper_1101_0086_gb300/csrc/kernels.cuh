@@ -173,9 +173,12 @@ template <typename T> __device__ __forceinline__ void kahan_add(T& s, T& c, T v)
 #ifndef MPA_L2PF_KC
 #define MPA_L2PF_KC 0
 #endif
-// the forward column pass (V_j, MPA_POST) reads what the row pass just
-// wrote; one wave ahead it gains 3.7 % (3815 -> 3957 GB/s on the 2^20 link,
-// split 2^12 x 2^8) while the inverse pass loses 6.6 % with it
+// the forward column passes (MPA_POST in the reverse mode's recompute, FWD in
+// levels with columns below 2^8) read what the row pass just wrote; one wave
+// ahead MPA_POST gains 3.7 % (3815 -> 3957 GB/s at 2^20, 2^12 x 2^8) while the
+// inverse pass loses 6.6 % with it.  FWD prefetches only where the node spectra
+// exceed L2 (129 MB): two intervals of 143 nodes at 2^17 x 2^7 columns 1075 ->
+// 1018 us, of 801 nodes at 2^15 858 -> 820, but 505 -> 512 at 2^16 x 143 (75 MB)
 #ifndef MPA_L2PF_KC_POST
 #define MPA_L2PF_KC_POST 304
 #endif
@@ -276,10 +279,11 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
         }
     }
 
-    constexpr int L2PF = MODE == KC_MPA_POST ? MPA_L2PF_KC_POST : MPA_L2PF_KC;
+    constexpr bool LEVEL_FWD = F == 0 && MODE == KC_FWD;  // (or a single field beyond 2^22: no error word)
+    constexpr int L2PF = MODE == KC_MPA_POST || LEVEL_FWD ? MPA_L2PF_KC_POST : MPA_L2PF_KC;
     if constexpr (FAST && L2PF > 0) {
         const long long tb = (long long)blockIdx.x + L2PF;
-        if (tb < (long long)gridDim.x) {
+        if (tb < (long long)gridDim.x && (!LEVEL_FWD || (p.err && p.ncols * L > (1ll << 24)))) {
             // the first node's columns of that tile (all of it when G <= N1)
             const long long col = tb * G;
             const int node = (int)(col >> p.logN1);
@@ -316,7 +320,7 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
             const long long c = (col0 + g) & N1m;
             unsigned long long th[XF::RL];
             if constexpr (FAST) phase_run<XF::RL>(c + (long long)j * p.N1, (long long)p.N1 * (L / XF::RL), p.flow, th);
-        [[maybe_unused]] C odd = mkc(T(0), T(0));
+            [[maybe_unused]] C odd = mkc(T(0), T(0));
 #pragma unroll
             for (int r = 0; r < XF::RL; ++r) {
                 const int row = j + r * (L / XF::RL);
