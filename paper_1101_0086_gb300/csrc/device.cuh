@@ -569,7 +569,7 @@ template <int L> struct TwDims {
 // up to 16 KB, bank conflicts and one CTA an SM less (us a step at 2^18 13.1 ->
 // 16.1, at 2^22 67 -> 85), so the two-level one holds lo - 1 instead of lo and
 // what FP32 leaves of hi = W_NHI^h (NHI <= 32): hi + (res + hi (lo - 1)), two
-// additions more than hi lo (13.6 and 68 us; 2^20 22.6 -> 23.3).
+// additions more than hi lo (13.4 and 68 us; 2^20 22.5 -> 23.2).
 template <typename T, int L, bool EX = false> struct Tw {
     static constexpr bool FULL = L >= 16 && (sizeof(T) == 8 ? L <= 2048 : EX && L <= 128);
     static constexpr bool COMP = EX && !FULL && L <= 2048;
@@ -578,32 +578,35 @@ template <typename T, int L, bool EX = false> struct Tw {
     static constexpr int N = FULL ? L : TwDims<L>::NLO + (COMP ? 2 : 1) * TwDims<L>::NHI;
 };
 
-// W_32^m in FP32 and what FP32 leaves of it, from the closed forms above.
-struct W32 {
-    float2 hi[32], res[32];
-};
-template <int M> constexpr double w32_cos() {
-    if constexpr (M > 16) return w32_cos<32 - M>();
-    else if constexpr (M % 8 == 0) return M == 0 ? 1.0 : M == 8 ? 0.0 : -1.0;
-    else if constexpr (M % 4 == 0) return M == 4 ? MPA_COS_PI_4 : -MPA_COS_PI_4;
-    else return Cs32<M>::c;
-}
-template <int M = 0> constexpr void w32_fill(W32& t) {
-    if constexpr (M < 32) {
-        constexpr double c = w32_cos<M>(), s = w32_cos<(M + 24) % 32>();  // sin x = cos(x - turn / 4)
-        t.hi[M].x = (float)c;
-        t.hi[M].y = (float)s;
-        t.res[M].x = (float)(c - (double)(float)c);
-        t.res[M].y = (float)(s - (double)(float)s);
-        w32_fill<M + 1>(t);
+// cos(2 pi m / 32) in FP32 and what FP32 leaves of it, from the closed forms
+// above: selected in registers (a table in constant memory costs each launch
+// cold, divergent reads: 0.2 us).
+template <int K> __host__ __device__ __forceinline__ void w32_pick(int k, float& hi, float& res) {
+    if constexpr (K < 8) {
+        constexpr double c = K == 4 ? MPA_COS_PI_4 : Cs32<K>::c;
+        constexpr float h = (float)c, r = (float)(c - (double)h);
+        hi = k == K ? h : hi;
+        res = k == K ? r : res;
+        w32_pick<K + 1>(k, hi, res);
     }
 }
-constexpr W32 w32_make() {
-    W32 t{};
-    w32_fill(t);
-    return t;
+__host__ __device__ __forceinline__ void w32_cos(int m, float& hi, float& res) {
+    m &= 31;
+    if (m > 16) m = 32 - m;
+    const int k = m > 8 ? 16 - m : m;  // the first quarter turn
+    hi = k == 0 ? 1.f : 0.f;
+    res = 0.f;
+    w32_pick<1>(k, hi, res);
+    if (m > 8) {
+        hi = -hi;
+        res = -res;
+    }
 }
-static __constant__ const W32 kW32 = w32_make();
+// W_32^m
+__host__ __device__ __forceinline__ void w32(int m, float2& hi, float2& res) {
+    w32_cos(m, hi.x, res.x);
+    w32_cos(m + 24, hi.y, res.y);  // sin x = cos(x - turn / 4)
+}
 
 // Slot of entry e of the low twiddle table.  A row-pass warp looks up
 // e = s j for 32 consecutive j and a power of two s; 8-byte entries sit in 16
@@ -617,7 +620,9 @@ template <int NLO> __host__ __device__ __forceinline__ int tw_lo_slot(int e) {
 
 template <typename T, int L, bool EX = false> __device__ __forceinline__ void tw_init(cx<T>* hi, cx<T>* lo, int tid, int nt) {
     typedef TwDims<L> D;
-    if constexpr (Tw<T, L, EX>::FULL) {
+    if constexpr (Tw<T, L, EX>::FULL && EX) {
+        for (int m = tid; m < L; m += nt) hi[m] = expi_ratio<T>(m, D::logL);
+    } else if constexpr (Tw<T, L, EX>::FULL) {
         // the first octant evaluated, the others its reflections (exact)
         for (int m = tid; m <= L / 8; m += nt) {
             const cx<T> w = expi_ratio<T>(m, D::logL);
@@ -633,13 +638,12 @@ template <typename T, int L, bool EX = false> __device__ __forceinline__ void tw
     } else if constexpr (Tw<T, L, EX>::COMP) {
         for (int i = tid; i < D::NLO + D::NHI; i += nt) {
             if (i < D::NLO) {
-                // cos x - 1 = -2 sin^2(x/2)
-                const T h = expi_ratio<T>(i, D::logL + 1).y;
-                lo[tw_lo_slot<D::NLO>(i)] = mkc(T(-2) * h * h, expi_ratio<T>(i, D::logL).y);
+                // cos x - 1 = -2 sin^2(x/2), sin x = 2 sin(x/2) cos(x/2)
+                const cx<T> w = expi_ratio<T>(i, D::logL + 1);
+                lo[tw_lo_slot<D::NLO>(i)] = mkc(T(-2) * w.y * w.y, T(2) * w.y * w.x);
             } else {
                 const int m = i - D::NLO;
-                hi[m] = kW32.hi[m * (32 / D::NHI)];
-                lo[D::NLO + m] = kW32.res[m * (32 / D::NHI)];
+                w32(m * (32 / D::NHI), hi[m], lo[D::NLO + m]);
             }
         }
     } else {
