@@ -171,7 +171,9 @@ MPA_API int mpa_plan_autotune(mpa_plan* plan, mpa_stream stream, int32_t* log2_n
  * CTA up to 2^14 FP32 / 2^13 FP64; for FP32 2^15 and 2^16 a cluster of 2 or
  * 4 CTAs exchanging through distributed shared memory).  It is the default
  * of FP32 plans up to 2^14; mpa_plan_autotune tries it first and reports it
- * as 0.
+ * as 0.  The split is the levels' (and, beyond 2^22 samples, the entry and exit
+ * transforms'); where its columns are longer than 2^max(8, log2(N) - 12) points,
+ * the reverse mode of an FP32 plan (mpa_adjoint) runs on columns of that length.
  * Host-only. */
 MPA_API int mpa_plan_set_split(mpa_plan* plan, int32_t log2_n2);
 

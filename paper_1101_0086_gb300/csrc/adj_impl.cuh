@@ -125,7 +125,8 @@ cudaError_t ssc_one(const SSCParams<T>& p, cudaStream_t st) {
     if (p.N1 % Gm::G != 0) return cudaErrorInvalidValue;
     const bool prof = g_prof_on.load(std::memory_order_relaxed);
     if (prof) prof_begin(st);
-    const cudaError_t el = launch_pdl(pdl_field<T>(p.N), ssc_kernel<T, L, MODE, F>, (unsigned)(p.N1 / Gm::G), Gm::NT, Gm::smem_bytes, st, p);
+    const cudaError_t el = launch_pdl(pdl_field<T>(p.N), ssc_kernel<T, L, MODE, F>, (unsigned)(p.N1 / Gm::G), Gm::NT,
+                                      Gm::smem_bytes, st, p);
     if (prof) prof_end(PK_KC_ADJ, st, 3.0 * (double)p.N * sizeof(cx<T>));
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return el;
@@ -146,7 +147,8 @@ cudaError_t ssr_one(const SSRParams<T>& p, cudaStream_t st) {
     if (p.nrows % Gm::G != 0) return cudaErrorInvalidValue;
     const bool prof = g_prof_on.load(std::memory_order_relaxed);
     if (prof) prof_begin(st);
-    const cudaError_t el = launch_pdl(pdl_field<T>(p.N), ssr_kernel<T, L, MODE, F>, (unsigned)(p.nrows / Gm::G), Gm::NT, Gm::smem_bytes, st, p);
+    const cudaError_t el = launch_pdl(pdl_field<T>(p.N), ssr_kernel<T, L, MODE, F>, (unsigned)(p.nrows / Gm::G), Gm::NT,
+                                      Gm::smem_bytes, st, p);
     if (prof) prof_end(PK_KR_ADJ, st, 3.0 * (double)p.nrows * L * sizeof(cx<T>));
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return el;

@@ -126,7 +126,9 @@ template <typename T> __device__ __forceinline__ T ksq(long long kk) {
 template <typename T> __host__ __device__ constexpr int kca_tiles(int L) { return sizeof(T) == 4 && L >= 1024 ? 2 : 0; }
 
 template <typename T, int L, int MODE>
-__global__ void __launch_bounds__(KCGeom<T, L, kca_tiles<T>(L)>::NT, KCGeom<T, L, kca_tiles<T>(L)>::NT <= 256 && sizeof(T) == 4 ? MPA_ADJ_MINB : 1) kca_kernel(const KCAParams<T> p) {
+__global__ void __launch_bounds__(KCGeom<T, L, kca_tiles<T>(L)>::NT,
+                                  KCGeom<T, L, kca_tiles<T>(L)>::NT <= 256 && sizeof(T) == 4 ? MPA_ADJ_MINB : 1)
+    kca_kernel(const KCAParams<T> p) {
     typedef cx<T> C;
     typedef KCGeom<T, L, kca_tiles<T>(L)> Gm;
     typedef typename Gm::P P;
@@ -231,7 +233,8 @@ __global__ void __launch_bounds__(KCGeom<T, L, kca_tiles<T>(L)>::NT, KCGeom<T, L
 }
 
 template <typename T, int L>
-__global__ void __launch_bounds__(KRGeom<T, L>::NT, KRGeom<T, L>::NT <= 256 && sizeof(T) == 4 ? MPA_ADJ_MINB_R : 1) kra_kernel(const KRAParams<T> p) {
+__global__ void __launch_bounds__(KRGeom<T, L>::NT, KRGeom<T, L>::NT <= 256 && sizeof(T) == 4 ? MPA_ADJ_MINB_R : 1)
+    kra_kernel(const KRAParams<T> p) {
     typedef cx<T> C;
     typedef KRGeom<T, L> Gm;
     typedef Tiling<T, 1> P;
@@ -480,7 +483,8 @@ template <typename T> struct SSRParams {
 };
 
 template <typename T, int L, int MODE, int F>
-__global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 256 && sizeof(T) == 4 ? MPA_ADJ_MINB : 1) ssc_kernel(const SSCParams<T> p) {
+__global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 256 && sizeof(T) == 4 ? MPA_ADJ_MINB : 1)
+    ssc_kernel(const SSCParams<T> p) {
     typedef cx<T> C;
     typedef KCGeom<T, L, F> Gm;
     typedef typename Gm::P P;
@@ -565,7 +569,8 @@ __global__ void __launch_bounds__(KCGeom<T, L, F>::NT, KCGeom<T, L, F>::NT <= 25
 }
 
 template <typename T, int L, int MODE, int F>
-__global__ void __launch_bounds__(KRGeom<T, L, F>::NT, KRGeom<T, L, F>::NT <= 256 && sizeof(T) == 4 ? MPA_ADJ_MINB_R : 1) ssr_kernel(const SSRParams<T> p) {
+__global__ void __launch_bounds__(KRGeom<T, L, F>::NT, KRGeom<T, L, F>::NT <= 256 && sizeof(T) == 4 ? MPA_ADJ_MINB_R : 1)
+    ssr_kernel(const SSRParams<T> p) {
     typedef cx<T> C;
     typedef KRGeom<T, L, F> Gm;
     typedef typename Gm::P P;

@@ -170,7 +170,8 @@ int run_group(mpa_batch* b, Group& g, cudaStream_t st) {
         for (long q = 0; q < g.n_int; ++q) {
             int rc = mpa_levels<T>(s, M, b->n_iter, g.active[(size_t)q], psi,
                                    g.has_work ? reinterpret_cast<cx<T>*>(b->ws + g.off_work) : nullptr, psi0c, state,
-                                   nodes, reinterpret_cast<const ScanNode*>(b->ws + g.off_scn), loff + (size_t)q * n, gain + (size_t)q * n, mon, 1, nullptr, st);
+                                   nodes, reinterpret_cast<const ScanNode*>(b->ws + g.off_scn), loff + (size_t)q * n,
+                                   gain + (size_t)q * n, mon, 1, nullptr, st);
             if (rc) return rc;
         }
     }

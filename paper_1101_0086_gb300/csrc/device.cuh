@@ -618,7 +618,8 @@ template <int NLO> __host__ __device__ __forceinline__ int tw_lo_slot(int e) {
     else return e;
 }
 
-template <typename T, int L, bool EX = false> __device__ __forceinline__ void tw_init(cx<T>* hi, cx<T>* lo, int tid, int nt) {
+template <typename T, int L, bool EX = false>
+__device__ __forceinline__ void tw_init(cx<T>* hi, cx<T>* lo, int tid, int nt) {
     typedef TwDims<L> D;
     if constexpr (Tw<T, L, EX>::FULL && EX) {
         for (int m = tid; m < L; m += nt) hi[m] = expi_ratio<T>(m, D::logL);
@@ -654,7 +655,8 @@ template <typename T, int L, bool EX = false> __device__ __forceinline__ void tw
     }
 }
 
-template <typename T, int L, bool EX> __device__ __forceinline__ cx<T> tw_get(const cx<T>* hi, const cx<T>* lo, int e) {
+template <typename T, int L, bool EX>
+__device__ __forceinline__ cx<T> tw_get(const cx<T>* hi, const cx<T>* lo, int e) {
     typedef TwDims<L> D;
     if constexpr (Tw<T, L, EX>::FULL) return hi[e];
     else if constexpr (Tw<T, L, EX>::COMP) {

@@ -123,7 +123,6 @@ template <typename T, int L, int F = 0> struct KCGeom {
     static constexpr int OHI = L > 32 ? L / 32 : 1;
     static constexpr size_t smem_elems = (size_t)TE + (TE >> P::PSH) + 1 + Tw<T, L, EX>::N +
                                          (size_t)G * (OLO + OHI);
-    // FP32: + the exp(2 pi i m/1024) table of the per-element phases
     static constexpr size_t smem_bytes = smem_elems * sizeof(cx<T>);
 };
 
@@ -1365,10 +1364,11 @@ template <bool STORE> __global__ void __launch_bounds__(SCAN_NT, 5) scan_pair_ke
 // the run's partial sums.  A thread per frequency leaves a short link with few
 // warps that each walk all M nodes one after another (N = 2^12: 16 blocks on
 // 152 SMs, bound by L2 latency); here every node of a panel is in flight at
-// once: FP32 20.9 -> 13.5 us at 2^12 x 143 nodes, 80 -> 43 us at 2^14 x 801.
-// Eight warps at 64 registers: four blocks an SM, whose load, sum and store
-// phases overlap (16 warps at 64 registers 52 us, at 101 registers 66 us on
-// the latter).
+// once: FP32 21.3 -> 13.2 us at 2^12 x 143 nodes, 21.0 -> 14.2 at 2^13 x 143,
+// 65.6 -> 22.2 at 2^12 x 801, 65.9 -> 27.0 at 2^13 x 801.  Eight warps at 64
+// registers (FP32 spills 48 bytes): four blocks an SM, whose load, sum and store
+// phases overlap (at 2^14 x 801, which takes the scan with phases since, 43 us;
+// 16 warps at 64 registers 52, at 101 registers 66).
 constexpr int SCS_W = 8;
 template <typename T>
 __global__ void __launch_bounds__(32 * SCS_W, sizeof(T) == 4 ? 4 : 2) scan_split_kernel(const ScanParams<T> p) {

@@ -19,7 +19,8 @@ static cudaError_t kn_one(const KNParams<double>& p, cudaStream_t st) {
     if (nblk <= 0) return cudaSuccess;
     const bool prof = g_prof_on.load(std::memory_order_relaxed);
     if (prof) prof_begin(st);
-    const cudaError_t el = launch_pdl(pdl_fills(nblk), kn_kernel<double, L, PIN, POUT>, (unsigned)nblk, Gm::NT, Gm::smem_bytes, st, p);
+    const cudaError_t el =
+        launch_pdl(pdl_fills(nblk), kn_kernel<double, L, PIN, POUT>, (unsigned)nblk, Gm::NT, Gm::smem_bytes, st, p);
     if (prof) {
         // every node read once and written once (a shared psi_0 once per link)
         const double cs = (double)sizeof(cx<double>), nodes = (double)p.nrows;

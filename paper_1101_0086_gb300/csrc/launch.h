@@ -83,8 +83,11 @@ inline cudaError_t launch_pdl(bool early, void (*kernel)(P...), dim3 grid, dim3 
 }
 // Whether a level's kernel of `blocks` blocks starts early: a grid that does
 // not fill the SMs twice over would be packed onto the first ones that fall
-// free (one span of a 2^12 link, 72 blocks of two node transforms and 128 of
-// the scan: 761 us with ordinary launches, 861 to 940 with early ones).
+// free.  Two intervals of three levels, ordinary / early, us: 2^13 x 143 nodes
+// (143 blocks of transforms, 256 of the scan) 185 / 201, one interval of 2^12 x
+// 801 (401, 128) 168 / 192, 2^13 x 801 (801, 256) 258 / 269.  At 2^12 x 143 (143
+// blocks of 256 threads, 128) early is the faster, 141 / 122; the line lies
+// where most grids gain.
 inline bool pdl_fills(long long blocks) {
     int sms = 0;
     return sm_count(&sms) == cudaSuccess && fills_twice(blocks, sms);

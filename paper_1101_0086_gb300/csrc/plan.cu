@@ -31,12 +31,6 @@ using namespace mpa::host;
 namespace mpa {
 namespace host {
 
-// One level-synchronous interval for nl links stored link-major (link l's
-// node j at psi + (l (M+1) + j) N, its psi_0 at psi0c + l N, its FP64 state
-// at state + l N).  loff[l] points link l's node constants for this
-// interval; gain[l] is its amplifier gain at the interval end (device).
-// Every iteration covers nodes 0..M of every link; node 0 always reads
-// psi_0, so V_0 (identical at every iteration) is simply recomputed.
 // Frequencies (N x links) from which the scan applies the phases of steps 2
 // and 5 (ScanParams::phases) instead of the node transforms' load and store.
 // A level in us, with / without: FP32, 143 nodes: 2^14 42.0 / 42.8, 2^15 83 /
@@ -46,6 +40,13 @@ namespace host {
 // 4134 / 4357.
 template <typename T> constexpr long long scan_phases_min() { return sizeof(T) == 4 ? 1ll << 14 : 1ll << 15; }
 
+// One level-synchronous interval for nl links stored link-major (link l's
+// node j at psi + (l (M+1) + j) N, its psi_0 at psi0c + l N, its FP64 state
+// at state + l N).  loff[l] points link l's node constants for this
+// interval; gain[l] is its amplifier gain at the interval end (device).
+// Every iteration covers nodes 0..M of every link; node 0 always reads
+// psi_0, so V_0 (identical at every iteration) is simply recomputed.
+//
 // With ph (many frequencies), psi holds A_hat_j before the node transforms
 // (level 0 reads psi_0 and applies the phases at the load) and F_j =
 // F[|A_j|^2 A_j] after them, and the scan turns F_j into the next level's
